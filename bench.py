@@ -55,6 +55,26 @@ CHAMFER_TRAFFIC_BYTES = {("batched_uneven", "k_tcpass", "eq1"): 7.72e9 + 5.41e9,
                          ("trajectory_50x50", "k_chamfer<false>", "eq2"): 19.57e6}
 
 
+def pruned_roof(points, queries, kernel_s, launch_pairs):
+    """Roofline entry of the pruned search (k_tree_search and k_tree_single). It evaluates the
+    direct form only for boxes of 8 points that the query's minimum so far does not exclude
+    (about 180 pairs per query on these clouds), so the 8-flop accounting of all pairs does not
+    apply to it. What it cannot do without are its bytes: every point read once (16 bytes) and a
+    (distance, index) record of 8 bytes per query."""
+    nbytes = 16 * points + 8 * queries
+    hbm = measured_peaks().get("hbm_gbs")
+    gbs = nbytes / kernel_s / 1e9 if kernel_s else None
+    return {"bound": "issue", "achieved": gbs, "peak": hbm, "unit": "GB/s",
+            "frac": gbs / hbm if (gbs and hbm) else None, "traffic": None,
+            "kernel": "k_tree_search + k_tree_single",
+            "kernel_ms": kernel_s * 1e3 if kernel_s else None,
+            "pairs_per_s_kernel": launch_pairs / kernel_s if kernel_s else None,
+            "accounting": "algorithmic bytes of the search against the measured copy bandwidth; "
+                          "pairs/s counts the (sim point, target) pairs that the minima are over, "
+                          "of which the search evaluates those its bounding boxes do not exclude "
+                          "(exactly: every result is that of all pairs)"}
+
+
 def measured_peaks():
     """The generated peak measurements of this machine's GPUs, if present."""
     try:
@@ -89,7 +109,7 @@ def parse():
     p.add_argument("--frames", type=int, default=None,
                    help="use only the first FRAMES frames of the trajectory (profiling runs)")
     p.add_argument("--shape", default=None,
-                   help="ENGINE:WARPS (tensor:0, tcgen05:0, direct:2): the nearest-neighbour "
+                   help="ENGINE:WARPS (pruned:0, tensor:0, tcgen05:0, direct:2): the nearest-neighbour "
                         "engine; batched_uneven plans with it instead of timing every shape")
     p.add_argument("--kernels-only", action="store_true",
                    help="batched_uneven: only the planned launch sequence (no plain per-frame "
@@ -497,6 +517,10 @@ def run_gpu(args, rank, world, dist):
                           f"{2 * FP32_LANES_PER_SM * sms * sm_max * 1e6 / 1e12:.1f} TFLOP/s",
             "kernel_ms": chamfer_avg_s * 1e3,
             "pairs_per_s_kernel": pairs / chamfer_avg_s if chamfer_n else None}
+    if engine == _lib.ENGINE_PRUNED:
+        roof = pruned_roof(T * (N + M), T * (N + (M if mode == _lib.BIDIR_MEAN else 0)),
+                           chamfer_avg_s, pairs)
+        achieved = None
     best_fma = max(fma.values()) / 1e12
     roof["peak_measured"] = {
         "scalar_fma_tflops": fma["scalar"] / 1e12, "packed_fma_tflops": fma["packed"] / 1e12,
@@ -735,6 +759,10 @@ def run_batched(args, rank, world, dist):
                           "both directions, against the FP32 CUDA-core FMA peak 2 x "
                           f"{FP32_LANES_PER_SM} lanes x {props.multi_processor_count} SMs x "
                           f"median SM clock under load ({sm_mhz:.0f} MHz; {sm_max:.0f} MHz max)"}
+    if shape[0] == "pruned":
+        pts = sum(int(t.n_off[-1]) + int(t.m_off[-1]) for t in trajs)
+        q = pts if mode == _lib.BIDIR_MEAN else sum(int(t.n_off[-1]) for t in trajs)
+        roof = pruned_roof(pts, q, ck, pairs)
     if tc:
         # the pass evaluates each pair once per direction on the tensor cores: one m16n8k16
         # MMA (4096 flop) per 128 pairs, in both directions for Eq. 1

@@ -221,15 +221,18 @@ int dc_batch_plan_async(const dc_frame* frames, int n_frames, int mode, void* ws
 int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream);
 
 /*
- * Tuning of the nearest-neighbour search. Three engines compute the same neighbours and losses
+ * Tuning of the nearest-neighbour search. Four engines compute the same neighbours and losses
  * (the float32 direct form, lowest index among equal distances):
+ *   DC_ENGINE_PRUNED -- the points of both clouds sorted along a space-filling curve, with
+ *     bounding boxes of runs of 8, 64 and 512 points; a query evaluates the direct form only for
+ *     boxes that its minimum so far does not exclude. Clouds of at most 2 097 152 points.
+ *     DC_ENGINE_AUTO takes it for calls (and batch plans) of at least 2.5e8 pairs, else the
+ *     direct engine.
  *   DC_ENGINE_TENSOR -- a tensor-core filter: the expanded form |p|^2 - 2 p.q + |q|^2 on
  *     split-fp16 operands, warp-level MMAs (16 points x 8 candidates each), keeps per point
  *     and quarter of the candidates the three best blocks of 128, and the direct form
  *     re-checks only the blocks that an error bound cannot exclude (every candidate when it
  *     cannot certify the blocks). Frames of at most 524 288 points per side.
- *     DC_ENGINE_AUTO takes it for calls (and batch plans) of at least 1e9 pairs and 5e7
- *     pairs per frame on average, where it pays back its fixed costs; else the direct engine.
  *   DC_ENGINE_TCGEN05 -- the same filter on tcgen05 MMAs (128 points x 128 candidates each)
  *     into tensor memory; same keys, same recovery, same results.
  *   DC_ENGINE_DIRECT -- every pair in the direct form on the CUDA cores; a CTA of w warps
@@ -240,7 +243,13 @@ int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream);
  * them per problem size and sets the winner before its calls); batch plans keep the choice
  * they were planned with.
  */
-enum { DC_ENGINE_AUTO = 0, DC_ENGINE_DIRECT = 1, DC_ENGINE_TENSOR = 2, DC_ENGINE_TCGEN05 = 3 };
+enum {
+    DC_ENGINE_AUTO = 0,
+    DC_ENGINE_DIRECT = 1,
+    DC_ENGINE_TENSOR = 2,
+    DC_ENGINE_TCGEN05 = 3,
+    DC_ENGINE_PRUNED = 4
+};
 
 typedef struct dc_tune {
     int32_t warps_per_cta; /* direct engine: 0 (automatic), 1, 2 or 4 */

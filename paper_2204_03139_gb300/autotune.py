@@ -1,8 +1,10 @@
 """Autotuner of the nearest-neighbour search's engine and tile shape.
 
 The shapes it chooses between:
+  ("pruned", 0)  the pruned search over sorted points and bounding boxes (clouds of at most
+                 2 097 152 points; the library's default for calls of 2.5e8 pairs and more);
   ("tensor", 0)  the tensor-core filter on warp-level MMAs (frames of at most 524 288
-                 points per side; the library's default for calls of 1e9 pairs and more);
+                 points per side);
   ("tcgen05", 0) the same filter on tcgen05 MMAs;
   ("direct", w)  the CUDA-core direct form with CTAs of w = 1, 2 or 4 warps (w x 512 sim
                  points held in registers; wide CTAs amortise the target staging and the
@@ -25,9 +27,9 @@ import torch
 
 from . import _lib
 
-SHAPES = (("tensor", 0), ("tcgen05", 0), ("direct", 1), ("direct", 2), ("direct", 4))
-_ENGINES = {"tcgen05": _lib.ENGINE_TCGEN05, "tensor": _lib.ENGINE_TENSOR,
-            "direct": _lib.ENGINE_DIRECT}
+SHAPES = (("pruned", 0), ("tensor", 0), ("tcgen05", 0), ("direct", 1), ("direct", 2), ("direct", 4))
+_ENGINES = {"pruned": _lib.ENGINE_PRUNED, "tcgen05": _lib.ENGINE_TCGEN05,
+            "tensor": _lib.ENGINE_TENSOR, "direct": _lib.ENGINE_DIRECT}
 WIDTHS = (1, 2, 4)
 _lock = threading.Lock()
 _cache: dict | None = None

@@ -64,7 +64,7 @@ Layout make_layout(const Sizes& s) {
     L.nnba = take(s.cols * 4);
     L.loss = take(s.n_frames * 4);
     L.part = take(s.n_frames * s.slices * 2 * 4);
-    L.frame_err = take(s.n_frames * 4);
+    L.frame_err = take(s.n_frames * 8);
     L.fbox = take(s.n_frames * 16);
     const long long tcp = s.tc_units > 0 ? s.rows + s.cols : 0;  // points with forms
     L.tc_ufr = take(s.tc_units * 4);
@@ -77,6 +77,17 @@ Layout make_layout(const Sizes& s) {
     L.kpart = take(s.tc_units > 0 ? s.tc_slots * 2 * TC_UNIT_ROWS * TC_KEYS * 4 : 0);
     L.tcfb = take(tcp * 4);
     L.tcfn = take(s.tc_units > 0 ? s.n_frames * 8 : 0);
+    const long long tp = s.tree ? s.rows + s.cols : 0;
+    L.step_frame = take(tp / TREE_STEP * 4);
+    L.tkey = take(tp * 4);
+    L.tord = take(tp * 4);
+    L.tcell = take(tp * 2);
+    L.tpts = take(tp * 16);
+    L.tkb = take(tp / 8 * 4);
+    L.tbox = take(tp / 8 * 32);
+    L.tbox1 = take(tp / 64 * 32);
+    L.tbox2 = take(tp / TREE_STEP * 32);
+    L.frec = take(s.tree ? s.sum_f * 48 : 0);
     L.total = off;
     return L;
 }
@@ -114,6 +125,17 @@ Ws make_ws(void* base, const Layout& L) {
     w.kpart = reinterpret_cast<unsigned*>(p + L.kpart);
     w.tcfb = reinterpret_cast<int*>(p + L.tcfb);
     w.tcfn = reinterpret_cast<int*>(p + L.tcfn);
+    w.step_frame = reinterpret_cast<int*>(p + L.step_frame);
+    w.tkey = reinterpret_cast<unsigned*>(p + L.tkey);
+    w.tqueue = reinterpret_cast<int*>(p + L.tord);
+    w.tord = reinterpret_cast<unsigned*>(p + L.tord);
+    w.tcell = reinterpret_cast<unsigned short*>(p + L.tcell);
+    w.tpts = reinterpret_cast<float*>(p + L.tpts);
+    w.tkb = reinterpret_cast<unsigned*>(p + L.tkb);
+    w.tbox = reinterpret_cast<float4*>(p + L.tbox);
+    w.tbox1 = reinterpret_cast<float4*>(p + L.tbox1);
+    w.frec = reinterpret_cast<float4*>(p + L.frec);
+    w.tbox2 = reinterpret_cast<float4*>(p + L.tbox2);
     return w;
 }
 
@@ -156,6 +178,7 @@ bool uniform_sizes(int T, int V, int F, int N, int M, Sizes& s, long long sub[3]
     // tensor-core regions, sized for both sides (the mode is not known here), when the frame
     // fits the key format; none for calls without targets
     s.tc_units = s.tc_slots = 0;
+    s.tree = with_tc && M > 0 && N <= TREE_MAX_POINTS && M <= TREE_MAX_POINTS ? 1 : 0;
     if (with_tc && M > 0 && Npad <= TC_MAX_COLS && Mpad <= TC_MAX_COLS) {
         const long long u0 = div_up(N, TC_UNIT_ROWS), u1 = div_up(M, TC_UNIT_ROWS);
         s.tc_units = (long long)T * (u0 + u1);
@@ -185,27 +208,26 @@ int check_ws(void* ws, size_t ws_bytes, size_t need) {
 
 int g_engine = ENGINE_AUTO;  // process-wide engine set by dc_tune_set
 
-// The Chamfer engine of a call: a tensor-core filter when the problem fits its key format
-// (tcgen05 by default, the warp-level MMA one when asked for), else, or when the direct
-// engine is requested, the CUDA-core direct form.
-// The default is the warp-level tensor-core filter for calls large enough to pay back its
-// fixed costs (candidate recovery, the fallback scans, the merge of split units): at least
-// 1e9 pairs and 5e7 per frame on average. Measured on one GB300 against the direct engine:
-// 1 frame of 32 768 points 329 vs 330 us, 10 frames of 10 000 282 vs 302 us, 40 frames of
-// 10 000 0.909 vs 1.028 ms, but 100 frames of 4096 497 vs 483 us and 1 frame of 16 384
-// 139 vs 119 us. The tcgen05 filter measured slower than the warp-level one on every
-// workload (at K = 16 each distance tile is one isolated tcgen05 MMA, whose issue and
-// synchronisation cost the folds cannot hide); it stays available on request.
-constexpr double TC_AUTO_MIN_PAIRS = 1e9;
-constexpr double TC_AUTO_MIN_FRAME_PAIRS = 5e7;
+// The Chamfer engine of a call: the one dc_tune_set asked for, when the problem fits it (else
+// the direct engine); by default the pruned search from TREE_AUTO_MIN_PAIRS pairs in all, and
+// the direct engine below, where the pruned search's sort and three launches take longer than
+// all pairs. Measured on one GB300, whole call with the gradient, replayed from a CUDA graph,
+// direct / warp-level tensor filter / pruned: 1 frame of 16 384 points 134 / 130 / 170 us and of
+// 32 768 377 / 317 / 200 us; 4 frames of 8192 110 / 117 / 109 us; 16 frames of 4096
+// 111 / 111 / 105 us and of 8192 302 / 255 / 151 us; 40 frames of 2048 94 / 102 / 110 us, of 4096
+// 217 / 207 / 151 us and of 16 384 2.56 / 1.87 / 0.56 ms; 100 frames of 1024 82 / 83 / 77 us.
+// The tensor-core filters, which evaluate every pair too, stay available on request (their
+// results are the same).
+// A pending stall test goes to the direct engine by default: the pruned search has no waits.
+constexpr double TREE_AUTO_MIN_PAIRS = 2.5e8;
 
-int choose_engine(bool tc_fits, double pairs, long long frames) {
+int choose_engine(bool tc_fits, bool tree_fits, double pairs) {
+    if (g_engine == ENGINE_TREE) return tree_fits ? ENGINE_TREE : ENGINE_DIRECT;
+    if (g_engine == ENGINE_AUTO)
+        return tree_fits && pairs >= TREE_AUTO_MIN_PAIRS && !stall_pending() ? ENGINE_TREE
+                                                                            : ENGINE_DIRECT;
     if (g_engine == ENGINE_DIRECT || !tc_fits) return ENGINE_DIRECT;
-    if (g_engine == ENGINE_TC5) return ENGINE_TC5;
-    if (g_engine == ENGINE_TC) return ENGINE_TC;
-    const bool big = pairs >= TC_AUTO_MIN_PAIRS &&
-                     pairs >= TC_AUTO_MIN_FRAME_PAIRS * (double)(frames > 0 ? frames : 1);
-    return big ? ENGINE_TC : ENGINE_DIRECT;
+    return g_engine;
 }
 
 int keyed_grid(int engine, long long chunks) {
@@ -222,7 +244,7 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     const bool chamfer = (phases & PH_CHAMFER) != 0;
     const int engine =
         chamfer && !direct_only
-            ? choose_engine(sz.tc_units > 0, (double)a.T * (double)a.N * (double)a.M, a.T)
+            ? choose_engine(sz.tc_units > 0, sz.tree != 0, (double)a.T * (double)a.N * (double)a.M)
             : ENGINE_DIRECT;
     const int warps =
         (chamfer && engine == ENGINE_DIRECT) ? choose_warps(a.mode, sub[2], sub[1], sub[0]) : 1;
@@ -240,6 +262,14 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     // with sampling to follow, the tables and the area CDFs (and the frame boxes of the
     // tensor-core forms) share one launch
     const bool fused = (phases & PH_AREA) && (phases & PH_SAMPLE);
+    if (engine == ENGINE_TREE) {
+        cudaError_t e = launch_tree(&a, w, T, a.pts ? 0 : a.F, std::max(a.N, a.M), rows, cols,
+                                    a.mode, st);
+        if (!e && epi_flags)
+            e = launch_epilogue(w, T, a.slices, a.grad ? a.V : 0, a.mode, epi_flags, loss_total,
+                                1, st);
+        return e ? cuda_fail(e, "kernel launch") : DC_OK;
+    }
     cudaError_t e = fused ? launch_build_area(a, w, st) : launch_build_uniform(a, w, st);
     if (!e && (phases & PH_AREA) && !fused) e = launch_area_cdf(w, T, st);
     if (!e && tc && !fused) e = launch_bbox(w, T, st);
@@ -266,7 +296,7 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     }
     if (!e && epi_flags)
         e = launch_epilogue(w, T, (int)sz.slices, a.grad ? a.V : 0, a.mode, epi_flags,
-                            loss_total, tc ? grid : 0, st);
+                            loss_total, tc ? 1 : 0, st);
     if (e) return cuda_fail(e, "kernel launch");
     return DC_OK;
 }
@@ -334,7 +364,7 @@ size_t direct_workspace_size(int T, int V, int F, int N, int M) {
 // ---- batch plans (host copy of what dc_batch_run needs to launch) ----
 struct Plan {
     Sizes sz;
-    int mode, any_grad, max_v, max_f, total_sub, n_units, warps, engine, tc_grid, tc_units;
+    int mode, any_grad, max_v, max_f, max_n, total_sub, n_units, warps, engine, tc_grid, tc_units;
     long long tc_chunks;
     size_t bytes;
 };
@@ -393,13 +423,14 @@ int dc_tune_set(const dc_tune* tune) {
     if (w != 0 && w != 1 && w != 2 && w != 4)
         return fail(DC_EINVAL, "warps_per_cta must be 0 (automatic), 1, 2 or 4");
     if (en != DC_ENGINE_AUTO && en != DC_ENGINE_DIRECT && en != DC_ENGINE_TENSOR &&
-        en != DC_ENGINE_TCGEN05)
+        en != DC_ENGINE_TCGEN05 && en != DC_ENGINE_PRUNED)
         return fail(DC_EINVAL, "engine must be DC_ENGINE_AUTO, DC_ENGINE_DIRECT, "
-                               "DC_ENGINE_TENSOR or DC_ENGINE_TCGEN05");
+                               "DC_ENGINE_TENSOR, DC_ENGINE_TCGEN05 or DC_ENGINE_PRUNED");
     set_tuned_warps(w);
     g_engine = en == DC_ENGINE_DIRECT    ? ENGINE_DIRECT
                : en == DC_ENGINE_TENSOR  ? ENGINE_TC
                : en == DC_ENGINE_TCGEN05 ? ENGINE_TC5
+               : en == DC_ENGINE_PRUNED  ? ENGINE_TREE
                                          : ENGINE_AUTO;
     return DC_OK;
 }
@@ -410,6 +441,7 @@ int dc_tune_get(dc_tune* tune) {
     tune->engine = g_engine == ENGINE_DIRECT ? DC_ENGINE_DIRECT
                    : g_engine == ENGINE_TC   ? DC_ENGINE_TENSOR
                    : g_engine == ENGINE_TC5  ? DC_ENGINE_TCGEN05
+                   : g_engine == ENGINE_TREE ? DC_ENGINE_PRUNED
                                              : DC_ENGINE_AUTO;
     return DC_OK;
 }
@@ -587,7 +619,7 @@ int dc_loss_traj_bwd(const float* verts, const int32_t* faces, const uint8_t* fa
 // batches
 // ---------------------------------------------------------------------------------------
 static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
-    s = Sizes{n, 0, 0, 0, 0, epilogue_slices(n), 0, 0};
+    s = Sizes{n, 0, 0, 0, 0, epilogue_slices(n), 0, 0, 1};
     sub[0] = sub[1] = sub[2] = 0;
     long long max_v = 0, tc_units = 0, tc_chunks = 0;
     bool tc_fits = true;
@@ -602,6 +634,7 @@ static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
         s.cols += Mpad;
         if (fr[k].grad_verts && fr[k].V > max_v) max_v = fr[k].V;
         tc_fits = tc_fits && Npad <= TC_MAX_COLS && Mpad <= TC_MAX_COLS;
+        if (fr[k].N > TREE_MAX_POINTS || fr[k].M > TREE_MAX_POINTS) s.tree = 0;
         const long long u0 = div_up(fr[k].N, TC_UNIT_ROWS), u1 = div_up(fr[k].M, TC_UNIT_ROWS);
         tc_units += u0 + u1;
         tc_chunks += u0 * (Mpad / TC_CHUNK) + u1 * (Npad / TC_CHUNK);
@@ -675,8 +708,11 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
         return fail(DC_EINVAL, "batch too large for 32-bit offsets");
     double pairs = 0.0;
     for (int k = 0; k < n_frames; ++k) pairs += (double)frames[k].N * (double)frames[k].M;
-    const int engine = choose_engine(sz.tc_units > 0, pairs, n_frames);
-    const int warps = engine == ENGINE_DIRECT ? choose_warps(mode, sub[2], sub[1], sub[0]) : 1;
+    const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, pairs);
+    // the pruned search's plans can run the direct engine too (stall tests)
+    const int warps = engine == ENGINE_DIRECT || engine == ENGINE_TREE
+                          ? choose_warps(mode, sub[2], sub[1], sub[0])
+                          : 1;
     const Layout L = make_layout(sz);
     // the staging image: the table regions [hdr, cdf), then the tensor-core unit tables
     const size_t img_bytes = L.cdf + (keyed(engine) ? L.tca - L.tc_ufr : 0);
@@ -707,7 +743,7 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
     int* turb = reinterpret_cast<int*>(tcimg.data() + (L.tc_urb - tc_beg));
     int* tupre = reinterpret_cast<int*>(tcimg.data() + (L.tc_upre - tc_beg));
     int tunit = 0, tchunk = 0;
-    int row0 = 0, col0 = 0, cdf0 = 0, unit = 0, subc = 0, any_grad = 0, max_v = 0, max_f = 0;
+    int row0 = 0, col0 = 0, cdf0 = 0, unit = 0, subc = 0, any_grad = 0, max_v = 0, max_f = 0, max_n = 0;
     // The table lists the frames largest first (N + M, ties in the caller's order). The
     // sampling and epilogue kernels run one CTA per (frame, slice) in table order, so the
     // long CTAs of big frames start first and the small ones fill in behind them instead of
@@ -767,6 +803,7 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
             subc += spu;
         }
         if (f.F > max_f) max_f = f.F;
+        max_n = std::max(max_n, std::max(f.N, f.M));
         if (f.grad_verts) {
             any_grad = 1;
             if (f.V > max_v) max_v = f.V;
@@ -817,6 +854,7 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
     p.any_grad = any_grad;
     p.max_v = max_v;
     p.max_f = max_f;
+    p.max_n = max_n;
     p.total_sub = subc;
     p.n_units = unit;
     p.warps = warps;
@@ -846,6 +884,15 @@ int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream) {
     const Layout L = make_layout(p.sz);
     const Ws w = make_ws(ws, L);
     const int n = (int)p.sz.n_frames, rows = (int)p.sz.rows, cols = (int)p.sz.cols;
+    if (p.engine == ENGINE_TREE && stall_pending()) p.engine = ENGINE_DIRECT;
+    if (p.engine == ENGINE_TREE) {
+        cudaError_t e = launch_tree(nullptr, w, n, p.max_f, p.max_n, rows, cols, p.mode, stream);
+        if (!e)
+            e = launch_epilogue(w, n, (int)p.sz.slices, p.any_grad ? p.max_v : 0, p.mode,
+                                EPI_RESCAN | EPI_LOSS | (p.any_grad ? EPI_GRAD : 0), loss_total,
+                                1, stream);
+        return e ? cuda_fail(e, "dc_batch_run") : DC_OK;
+    }
     const bool tc = keyed(p.engine);
     cudaError_t e = launch_reset(w, stream);
     if (!e) e = launch_area_cdf(w, n, stream);  // and the frame boxes
@@ -857,7 +904,7 @@ int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream) {
     if (!e)
         e = launch_epilogue(w, n, (int)p.sz.slices, p.any_grad ? p.max_v : 0, p.mode,
                             EPI_RESCAN | EPI_LOSS | (p.any_grad ? EPI_GRAD : 0), loss_total,
-                            tc ? p.tc_grid : 0, stream);
+                            tc ? 1 : 0, stream);
     if (e) return cuda_fail(e, "dc_batch_run");
     return DC_OK;
 }

@@ -442,6 +442,7 @@ int choose_warps(int mode, long long sub_w4, long long sub_w2, long long sub_w1)
 }
 
 int take_stall() { return g_stall_next.exchange(0); }
+bool stall_pending() { return g_stall_next.load() != 0; }
 
 cudaError_t launch_chamfer(const Ws& w, int n_units, int total_sub, int mode, int warps,
                            cudaStream_t s) {

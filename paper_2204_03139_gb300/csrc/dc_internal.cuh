@@ -115,8 +115,18 @@ static_assert(TC_BLOCK % TC_ROWS_PER_WARP == 0 || TC_ROWS_PER_WARP % TC_BLOCK ==
               "a warp's rows are part of a block or whole blocks");
 
 // ENGINE_TC: the filter on warp-level MMAs; ENGINE_TC5: on tcgen05 MMAs into tensor memory.
-// Both write the same keys, which the same kernels merge and resolve.
-enum : int { ENGINE_AUTO = 0, ENGINE_DIRECT = 1, ENGINE_TC = 2, ENGINE_TC5 = 3 };
+// Both write the same keys, which the same kernels merge and resolve. ENGINE_TREE: the pruned
+// search over sorted points and bounding boxes (tree.cu).
+enum : int {
+    ENGINE_AUTO = 0,
+    ENGINE_DIRECT = 1,
+    ENGINE_TC = 2,
+    ENGINE_TC5 = 3,
+    ENGINE_TREE = 4
+};
+constexpr int TREE_STEP = 256;  // queries per CTA of the pruned search (frames start at multiples)
+constexpr int TREE_MAX_POINTS = 1 << 21;  // points per side (index bits beside a key's low bits)
+static_assert(ROW_PAD % TREE_STEP == 0 && COL_PAD % TREE_STEP == 0, "steps lie in one frame");
 __host__ __device__ inline bool keyed(int engine) {
     return engine == ENGINE_TC || engine == ENGINE_TC5;
 }
@@ -179,14 +189,15 @@ struct WsHeader {
     int tc_total;     // their chunks of TC_CHUNK columns (live frames only)
     int tc_fallback;  // rows whose keys certified no candidate set (scanned in full)
     int tc_next;      // next unit to take, when the pass hands out whole units on demand
-    int pad[46];
+    int tree_n;       // pruned search: queued queries
+    int pad[45];
 };
 
 // Byte offsets of every region of a workspace (computed on the host).
 struct Layout {
     size_t hdr, frames, rowpre, colpre, unit_frame, unit_rb, unit_pre, cdf, x, fw, tsoa, tpl,
         pab, pba, nnab, nnba, loss, part, frame_err, fbox, tc_ufr, tc_urb, tc_upre, tca, tcb,
-        kab, kba, kpart, tcfb, tcfn, total;
+        kab, kba, kpart, tcfb, tcfn, step_frame, tkey, tord, tcell, tpts, tkb, tbox, tbox1, tbox2, frec, total;
 };
 
 struct Sizes {
@@ -194,6 +205,7 @@ struct Sizes {
     long long slices;    // epilogue slices per frame
     long long tc_units;  // tensor-core units (0: no tensor-core regions)
     long long tc_slots;  // CTAs the partial-key buffer is sized for
+    long long tree;      // 1: regions of the pruned search
 };
 
 // Epilogue slices per frame: as many as keep all (frame, slice) CTAs in one wave, at most
@@ -224,7 +236,8 @@ struct Ws {
     int* nnab;         // [rows] fallback neighbour buffers
     int* nnba;         // [cols]
     float* loss;       // [n_frames] fallback loss buffer
-    int* frame_err;    // [n_frames] error code of the fused build + area launch, per frame
+    int* frame_err;    // [n_frames][2] error code of the fused build + area launch, per frame,
+                       // or of the pruned search's preparation, per frame and side
     float* part;       // [n_frames][slices][2] loss partial sums
     float4* fbox;      // [n_frames] (centre x, y, z, scale) of the tensor-core forms
     int* tc_ufr;       // [tc_units] frame of each tensor-core unit
@@ -238,6 +251,19 @@ struct Ws {
     int* tcfb;         // [rows + cols] frame-local indices of the rows the keys did not
                        // certify, each frame's list at its own row (rows + column) range
     int* tcfn;         // [n_frames][2] lengths of those lists (zeroed by the staging)
+    // pruned search: sim points then targets, padded as the rows and columns
+    int* step_frame;           // [(rows + cols) / TREE_STEP] frame of every step
+    unsigned* tkey;            // [rows + cols] curve key of every point; after the preparation
+                               // in sorted order
+    unsigned* tord;            // [rows + cols] (low key bits, index) in counting-sort order
+    unsigned short* tcell;     // [rows + cols] and the counting-sort cell
+    int* tqueue;               // queries searched one at a time (the region of tord)
+    float* tpts;               // [rows + cols][4] sorted blocks of 8: x[8] y[8] z[8] index[8]
+    unsigned* tkb;             // [(rows + cols) / 8] first key of every block
+    float4* tbox;              // [(rows + cols) / 8][2] (lo, hi) of 8 points
+    float4* tbox1;             // [(rows + cols) / 64][2] of 64
+    float4* frec;              // [sum F][3] corners of every face, per frame (sampled frames)
+    float4* tbox2;             // [(rows + cols) / TREE_STEP][2] of 512 (from the frame's start)
 };
 
 Ws make_ws(void* base, const Layout& L);
@@ -345,11 +371,16 @@ int choose_warps(int mode, long long sub_w4, long long sub_w2, long long sub_w1)
 void set_tuned_warps(int warps);  // 0: automatic
 void inject_stall();              // the next Chamfer launch never gets its first chunk
 int take_stall();                 // 1 once after inject_stall (read by the Chamfer launchers)
+bool stall_pending();
+// the pruned search: preparation (a = nullptr: the frame table is in the workspace) and search,
+// leaving (distance bits << 32 | index) in pab (and pba in Eq. 1)
+cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max_f, int max_n,
+                        int rows, int cols, int mode, cudaStream_t s);
 int tuned_warps();
 // epilogue: neighbour recovery (rescan), loss partials, gradient scatter
 enum : int { EPI_RESCAN = 1, EPI_LOSS = 2, EPI_GRAD = 4 };
 cudaError_t launch_epilogue(const Ws& w, int n_frames, int slices, int max_v, int mode,
-                            int flags, float* total, int tc_grid, cudaStream_t s);
+                            int flags, float* total, int exact, cudaStream_t s);
 // sum_t w_t L_t of given per-frame losses, in the fixed order of the trajectory calls
 cudaError_t launch_loss_total(const float* lf, const float* w, int T, float* total,
                               cudaStream_t s);

@@ -42,7 +42,7 @@ struct EpiArgs {
     int flags;     // EPI_RESCAN | EPI_LOSS | EPI_GRAD
     int bidir;
     int use_smem;  // one slice per frame and the V x 3 accumulator fits in shared memory
-    int exact;     // the packed minima hold the neighbour's index itself (tensor-core path)
+    int exact;     // the packed minima hold the neighbour's index itself (all but the direct engine)
 };
 
 __device__ __forceinline__ float block_sum_fixed(float v, float* s_red) {
@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
     const float* PX = w.tpl + 3LL * col0;  // compact target planes X[Mpad], Y, Z
     const float* PY = PX + fr->Mpad;
     const float* PZ = PY + fr->Mpad;
+    const float* tgt = fr->tgt;  // as given: the exact mode (the pruned search stages no planes)
     const int i0 = (int)((long long)N * sl / e.slices);
     const int i1 = (int)((long long)N * (sl + 1) / e.slices);
     const bool exact = e.exact != 0 && rescan;
@@ -156,9 +157,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
                 for (int r = 0; r < 2; ++r) {
                     fr4[r] = make_int4(-1, 0, 0, 0);
                     if (nr[r] >= 0) {
-                        yr[r][0] = __ldg(&PX[nr[r]]);
-                        yr[r][1] = __ldg(&PY[nr[r]]);
-                        yr[r][2] = __ldg(&PZ[nr[r]]);
+                        yr[r][0] = __ldg(&tgt[3LL * nr[r]]);
+                        yr[r][1] = __ldg(&tgt[3LL * nr[r] + 1]);
+                        yr[r][2] = __ldg(&tgt[3LL * nr[r] + 2]);
                         fr4[r] = __ldg(&w.fw[row0 + ir[r]]);
                     }
                 }
@@ -269,9 +270,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
                     vr[r] = jr[r] < j1;
                     const int jj = vr[r] ? jr[r] : j0;
                     pr[r] = vr[r] ? __ldg(&w.pba[col0 + jj]) : EMPTY;
-                    tr[r][0] = __ldg(&PX[jj]);
-                    tr[r][1] = __ldg(&PY[jj]);
-                    tr[r][2] = __ldg(&PZ[jj]);
+                    tr[r][0] = __ldg(&tgt[3LL * jj]);
+                    tr[r][1] = __ldg(&tgt[3LL * jj + 1]);
+                    tr[r][2] = __ldg(&tgt[3LL * jj + 2]);
                 }
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
@@ -481,7 +482,7 @@ int g_smem_limit[64];
 constexpr int EPI_THREADS_ONE_SLICE = 4 * EPI_THREADS;
 
 cudaError_t launch_epilogue(const Ws& w, int n_frames, int slices, int max_v, int mode,
-                            int flags, float* total, int tc_grid, cudaStream_t s) {
+                            int flags, float* total, int exact, cudaStream_t s) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
@@ -499,7 +500,7 @@ cudaError_t launch_epilogue(const Ws& w, int n_frames, int slices, int max_v, in
     a.slices = slices;
     a.flags = flags;
     a.bidir = mode == DC_BIDIR_MEAN;
-    a.exact = tc_grid > 0;
+    a.exact = exact;
     const bool grad = (flags & EPI_GRAD) && max_v > 0;
     const size_t need = (size_t)max_v * 3 * sizeof(float);
     a.use_smem = grad && slices == 1 && need <= (size_t)g_smem_limit[dev];

@@ -2,7 +2,7 @@
 #include <cuda_fp16.h>
 #include <math.h>
 
-#include "dc_internal.cuh"
+#include "dc_sampling.cuh"
 
 namespace dc {
 
@@ -10,38 +10,6 @@ namespace {
 
 constexpr float ROW_SENTINEL = 1e18f;   // coordinate of padded sim points
 constexpr float COL_SENTINEL = -1e18f;  // coordinate of padded target points
-
-__device__ __forceinline__ void set_status(int* st, int code) { atomicCAS(st, DC_OK, code); }
-
-// largest k in [0, n) with pre[k] <= g (pre is non-decreasing, pre[0] = 0)
-__device__ __forceinline__ int last_le(const int* pre, int n, int g) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (pre[mid] <= g)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ bool coord_ok(float v) { return fabsf(v) <= COORD_MAX; }
-
-// Frame k's weight w_t in the total and the multiplier of its gradient. The forward uses w_t
-// for both. The recomputing backward gets the objective's derivatives: g_t = dJ/dL_t =
-// w_t dJ/dL_total + dJ/dL_t(direct), and 0 for a frame of weight 0, whose forward L_t is the
-// constant 0.
-__device__ __forceinline__ void frame_scales(const UniformArgs& a, int k, float& w, float& gs) {
-    w = a.weight ? a.weight[k] : 1.0f;
-    if (a.bwd) {
-        const float gt = a.gtotal ? a.gtotal[0] : 0.0f;
-        const float gf = a.gframes ? a.gframes[k] : 0.0f;
-        gs = w == 0.0f ? 0.0f : __fadd_rn(__fmul_rn(w, gt), gf);
-    } else {
-        gs = w;
-    }
-}
 
 // ---------------------------------------------------------------------------------------
 // tensor-core forms (see dc_internal.cuh): frame box, centre and scale, and the A / B forms
@@ -174,32 +142,8 @@ __device__ void build_uniform(const UniformArgs& a, const Ws& w) {
         const int k = k0 + tid;
         bool live = false;
         if (k < a.T) {
-            FrameDesc f;
-            f.verts = a.verts ? a.verts + 3LL * k * a.V : nullptr;
-            f.faces = a.faces;
-            f.mask = a.mask;
-            f.draws = a.draws ? a.draws + 3LL * k * a.N : nullptr;
-            f.pts = a.pts ? a.pts + 3LL * k * a.N : nullptr;
-            f.tgt = a.tgt ? a.tgt + 3LL * k * a.M : nullptr;
-            f.loss = a.loss ? a.loss + k : w.loss + k;
-            f.nn_ab = a.nn_ab ? a.nn_ab + (long long)k * a.N : w.nnab + (long long)k * Npad;
-            f.nn_ba = a.nn_ba ? a.nn_ba + (long long)k * a.M : w.nnba + (long long)k * Mpad;
-            f.grad = a.grad ? a.grad + 3LL * k * a.V : nullptr;
-            f.out_pts = a.out_pts ? a.out_pts + 3LL * k * a.N : nullptr;
-            f.out_face = a.out_face ? a.out_face + (long long)k * a.N : nullptr;
-            f.out_bary = a.out_bary ? a.out_bary + 3LL * k * a.N : nullptr;
-            f.V = a.V;
-            f.F = a.F;
-            f.N = a.N;
-            f.M = a.M;
-            f.Npad = Npad;
-            f.Mpad = Mpad;
-            frame_scales(a, k, f.weight, f.gscale);
-            f.skip = f.weight == 0.0f || f.gscale == 0.0f;
+            FrameDesc f = uniform_frame(a, w, k);
             live = !f.skip;
-            f.row0 = k * Npad;
-            f.col0 = k * Mpad;
-            f.cdf0 = k * a.F;
             f.unit0 = 0;  // set below: live frames before this one
             w.frames[k] = f;
             w.rowpre[k] = k * Npad;
@@ -292,88 +236,6 @@ __global__ void __launch_bounds__(BUILD_THREADS) k_build_uniform(UniformArgs a, 
     pdl_entry();
     build_uniform(a, w);
 }
-
-// ---------------------------------------------------------------------------------------
-// area CDF: two-float (compensated) prefix sum of the float32 face areas, so that the
-// stored C_f is the float32 rounding of the exact prefix sum of those areas
-// ---------------------------------------------------------------------------------------
-struct FF {
-    float hi, lo;
-};
-
-__device__ __forceinline__ FF ff_norm(float s, float e) {
-    float h = __fadd_rn(s, e);
-    return {h, __fsub_rn(e, __fsub_rn(h, s))};
-}
-
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
-__device__ __forceinline__ FF ff_add(FF a, FF b) {
-    float s, e;
-    two_sum(a.hi, b.hi, s, e);
-    return ff_norm(s, __fadd_rn(e, __fadd_rn(a.lo, b.lo)));
-}
-
-__device__ __forceinline__ FF ff_add1(FF a, float b) {
-    float s, e;
-    two_sum(a.hi, b, s, e);
-    return ff_norm(s, __fadd_rn(e, a.lo));
-}
-
-// area of face f = 1/2 |(p1 - p0) x (p2 - p0)|; flags bad indices / coordinates
-__device__ __forceinline__ float face_area(const float* __restrict__ verts,
-                                           const int* __restrict__ faces, int V, int f,
-                                           bool& bad_idx, bool& bad_val) {
-    const int i0 = faces[3 * f], i1 = faces[3 * f + 1], i2 = faces[3 * f + 2];
-    if ((unsigned)i0 >= (unsigned)V || (unsigned)i1 >= (unsigned)V ||
-        (unsigned)i2 >= (unsigned)V) {
-        bad_idx = true;
-        return 0.0f;
-    }
-    const float* p0 = verts + 3LL * i0;
-    const float* p1 = verts + 3LL * i1;
-    const float* p2 = verts + 3LL * i2;
-    float q[9] = {p0[0], p0[1], p0[2], p1[0], p1[1], p1[2], p2[0], p2[1], p2[2]};
-#pragma unroll
-    for (int k = 0; k < 9; ++k) bad_val |= !coord_ok(q[k]);
-    // explicit roundings: both passes of the scan must see bit-identical areas
-    const float e1x = __fsub_rn(q[3], q[0]), e1y = __fsub_rn(q[4], q[1]),
-                e1z = __fsub_rn(q[5], q[2]);
-    const float e2x = __fsub_rn(q[6], q[0]), e2y = __fsub_rn(q[7], q[1]),
-                e2z = __fsub_rn(q[8], q[2]);
-    const float cx = __fsub_rn(__fmul_rn(e1y, e2z), __fmul_rn(e1z, e2y));
-    const float cy = __fsub_rn(__fmul_rn(e1z, e2x), __fmul_rn(e1x, e2z));
-    const float cz = __fsub_rn(__fmul_rn(e1x, e2y), __fmul_rn(e1y, e2x));
-    const float n2 = __fmaf_rn(cz, cz, __fmaf_rn(cy, cy, __fmul_rn(cx, cx)));
-    return __fmul_rn(0.5f, __fsqrt_rn(n2));
-}
-
-// The area weight of face f: its area, or 0 for a face outside the sampled subset
-// (Sec. IV-F). The face is still checked, so that bad indices are reported either way.
-__device__ __forceinline__ float face_weight(const float* __restrict__ verts,
-                                             const int* __restrict__ faces,
-                                             const uint8_t* __restrict__ mask, int V, int f,
-                                             bool& bad_idx, bool& bad_val) {
-    const float a = face_area(verts, faces, V, f, bad_idx, bad_val);
-    return (mask && mask[f] == 0) ? 0.0f : a;
-}
-
-constexpr int CDF_THREADS = 1024;
-
-// What the area step needs to know about one frame.
-struct AreaFrame {
-    const float* verts;   // [V][3]
-    const int* faces;     // [F][3]
-    const uint8_t* mask;  // [F] nullable
-    float* grad;          // [V][3] nullable: zeroed here for the epilogue's accumulation
-    float* cdf;           // [F] out
-    int F, V;
-    bool skip;            // weight 0: only the gradient (zero) is written
-};
 
 // One block (CDF_THREADS threads) computes one frame's area CDF; errors go to *err with
 // atomicCAS(DC_OK -> code), so the first one stays.
@@ -505,41 +367,16 @@ __device__ __forceinline__ void sample_row(const Ws& w, const FrameDesc* fr, int
             if (!(rf >= 0.0f && rf <= 1.0f && r1 >= 0.0f && r1 <= 1.0f && r2 >= 0.0f &&
                   r2 <= 1.0f))
                 set_status(&w.hdr->status, DC_EINVAL);
-            const int F = fr->F;
-            const float t = __fmul_rn(rf, cdf[F - 1]);
-            int lo = 0, hi = F;  // first f with cdf[f] > t
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (cdf[mid] > t)
-                    hi = mid;
-                else
-                    lo = mid + 1;
-            }
-            const int f = min(lo, F - 1);
-            const int i0 = fr->faces[3 * f], i1 = fr->faces[3 * f + 1], i2 = fr->faces[3 * f + 2];
-            const int V = fr->V;
-            if ((unsigned)i0 < (unsigned)V && (unsigned)i1 < (unsigned)V &&
-                (unsigned)i2 < (unsigned)V) {
-                const float* p0 = fr->verts + 3LL * i0;
-                const float* p1 = fr->verts + 3LL * i1;
-                const float* p2 = fr->verts + 3LL * i2;
-                const float s = __fsqrt_rn(r1);
-                const float w0 = __fsub_rn(1.0f, s);
-                const float w1 = __fmul_rn(s, __fsub_rn(1.0f, r2));
-                const float w2 = __fmul_rn(s, r2);
-                x.x = __fmaf_rn(w2, p2[0], __fmaf_rn(w1, p1[0], __fmul_rn(w0, p0[0])));
-                x.y = __fmaf_rn(w2, p2[1], __fmaf_rn(w1, p1[1], __fmul_rn(w0, p0[1])));
-                x.z = __fmaf_rn(w2, p2[2], __fmaf_rn(w1, p1[2], __fmul_rn(w0, p0[2])));
-                q = make_int4(f, __float_as_int(w0), __float_as_int(w1), __float_as_int(w2));
+            if (pick_point(cdf, fr->F, fr->V, fr->verts, fr->faces, rf, r1, r2, x, q)) {
+                const int f = q.x;
                 if (fr->out_face) fr->out_face[i] = f;
                 if (fr->out_bary) {
-                    fr->out_bary[3LL * i] = w0;
-                    fr->out_bary[3LL * i + 1] = w1;
-                    fr->out_bary[3LL * i + 2] = w2;
+                    fr->out_bary[3LL * i] = __int_as_float(q.y);
+                    fr->out_bary[3LL * i + 1] = __int_as_float(q.z);
+                    fr->out_bary[3LL * i + 2] = __int_as_float(q.w);
                 }
             } else {
                 set_status(&w.hdr->status, DC_EINVAL);
-                x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
             if (fr->out_pts) {
                 fr->out_pts[3LL * i] = x.x;
