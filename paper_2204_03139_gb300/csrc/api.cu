@@ -80,8 +80,8 @@ Layout make_layout(const Sizes& s) {
     const long long tp = s.tree ? s.rows + s.cols : 0;
     L.step_frame = take(tp / TREE_STEP * 4);
     L.tkey = take(tp * 4);
-    L.tord = take(tp * 4);
-    L.tcell = take(tp * 2);
+    L.tord = take(tp * 8);
+    L.y = take(s.tree ? s.cols * 16 : 0);
     L.tpts = take(tp * 16);
     L.tkb = take(tp / 8 * 4);
     L.tbox = take(tp / 8 * 32);
@@ -128,8 +128,8 @@ Ws make_ws(void* base, const Layout& L) {
     w.step_frame = reinterpret_cast<int*>(p + L.step_frame);
     w.tkey = reinterpret_cast<unsigned*>(p + L.tkey);
     w.tqueue = reinterpret_cast<int*>(p + L.tord);
-    w.tord = reinterpret_cast<unsigned*>(p + L.tord);
-    w.tcell = reinterpret_cast<unsigned short*>(p + L.tcell);
+    w.tord = reinterpret_cast<unsigned long long*>(p + L.tord);
+    w.y = reinterpret_cast<float4*>(p + L.y);
     w.tpts = reinterpret_cast<float*>(p + L.tpts);
     w.tkb = reinterpret_cast<unsigned*>(p + L.tkb);
     w.tbox = reinterpret_cast<float4*>(p + L.tbox);

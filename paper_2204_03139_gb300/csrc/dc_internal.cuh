@@ -197,7 +197,7 @@ struct WsHeader {
 struct Layout {
     size_t hdr, frames, rowpre, colpre, unit_frame, unit_rb, unit_pre, cdf, x, fw, tsoa, tpl,
         pab, pba, nnab, nnba, loss, part, frame_err, fbox, tc_ufr, tc_urb, tc_upre, tca, tcb,
-        kab, kba, kpart, tcfb, tcfn, step_frame, tkey, tord, tcell, tpts, tkb, tbox, tbox1, tbox2, frec, total;
+        kab, kba, kpart, tcfb, tcfn, step_frame, y, tkey, tord, tpts, tkb, tbox, tbox1, tbox2, frec, total;
 };
 
 struct Sizes {
@@ -255,8 +255,8 @@ struct Ws {
     int* step_frame;           // [(rows + cols) / TREE_STEP] frame of every step
     unsigned* tkey;            // [rows + cols] curve key of every point; after the preparation
                                // in sorted order
-    unsigned* tord;            // [rows + cols] (low key bits, index) in counting-sort order
-    unsigned short* tcell;     // [rows + cols] and the counting-sort cell
+    float4* y;                 // [cols] targets as given (w lane unused)
+    unsigned long long* tord;  // [rows + cols] cell, low key bits, index in counting-sort order
     int* tqueue;               // queries searched one at a time (the region of tord)
     float* tpts;               // [rows + cols][4] sorted blocks of 8: x[8] y[8] z[8] index[8]
     unsigned* tkb;             // [(rows + cols) / 8] first key of every block

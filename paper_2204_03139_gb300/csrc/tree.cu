@@ -245,24 +245,35 @@ __device__ void tree_scan_cdf(float* cdf, int F, int* err) {
     __syncthreads();
 }
 
-// Area weight of face f and its three corners q[9] (zeros, and weight 0, for a face with an
-// index out of range; bad is set for it and for coordinates out of range).
-__device__ __forceinline__ float face_record(const float* __restrict__ verts,
+// Area weights of two faces and their corners q[9] (zeros, and weight 0, for a face with an index
+// out of range; bad is set for it and for coordinates out of range); the loads of both overlap.
+__device__ __forceinline__ void face_record2(const float* __restrict__ verts,
                                              const int* __restrict__ faces,
-                                             const uint8_t* __restrict__ mask, int V, int f,
-                                             float (&q)[9], bool& bad) {
-    const int i0 = faces[3 * f], i1 = faces[3 * f + 1], i2 = faces[3 * f + 2];
-    if ((unsigned)i0 >= (unsigned)V || (unsigned)i1 >= (unsigned)V || (unsigned)i2 >= (unsigned)V) {
-        bad = true;
+                                             const uint8_t* __restrict__ mask, int V,
+                                             const int (&f)[2], float (&q)[2][9], float (&A)[2],
+                                             bool& bad) {
+    int v[2][3];
+    bool in[2];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) q[k] = 0.0f;
-        return 0.0f;
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[h][c] = __ldg(faces + 3 * f[h] + c);
+        in[h] = (unsigned)v[h][0] < (unsigned)V && (unsigned)v[h][1] < (unsigned)V &&
+                (unsigned)v[h][2] < (unsigned)V;
+        bad |= !in[h];
     }
-    const float *p0 = verts + 3LL * i0, *p1 = verts + 3LL * i1, *p2 = verts + 3LL * i2;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) q[k] = p0[k], q[3 + k] = p1[k], q[6 + k] = p2[k];
-    const float A = corner_area(q, bad);
-    return (mask && mask[f] == 0) ? 0.0f : A;
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                q[h][3 * c + k] = in[h] ? __ldg(verts + 3LL * v[h][c] + k) : 0.0f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        A[h] = corner_area(q[h], bad);
+        if (mask && mask[f[h]] == 0) A[h] = 0.0f;
+    }
 }
 
 // pick_face of two draws at once: their binary searches' dependent loads overlap
@@ -406,17 +417,22 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
     if (sampled) {
         if (S > 1) cl.sync();  // every CTA of the cluster runs: its shared memory may be written
         const int fa = (int)((long long)fr.F * r / S), fb = (int)((long long)fr.F * (r + 1) / S);
-        for (int f = fa + tid; f < fb; f += PREP_THREADS) {
-            float q[9];
-            const float A = face_record(fr.verts, fr.faces, fr.mask, fr.V, f, q, bad);
-            rec[3 * f] = make_float4(q[0], q[1], q[2], q[3]);
-            rec[3 * f + 1] = make_float4(q[4], q[5], q[6], q[7]);
-            rec[3 * f + 2] = make_float4(q[8], 0.f, 0.f, 0.f);
-            if (cdf_shared) {
+        for (int fs = fa + tid; fs < fb; fs += 2 * PREP_THREADS) {
+            const int ff[2] = {fs, min(fs + PREP_THREADS, fb - 1)};  // the last may be done twice
+            float q[2][9], A[2];
+            face_record2(fr.verts, fr.faces, fr.mask, fr.V, ff, q, A, bad);
 #pragma unroll
-                for (int c = 0; c < S; ++c) remote(cdf, c)[f] = A;
-            } else {
-                cdf[f] = A;
+            for (int h = 0; h < 2; ++h) {
+                const int f = ff[h];
+                rec[3 * f] = make_float4(q[h][0], q[h][1], q[h][2], q[h][3]);
+                rec[3 * f + 1] = make_float4(q[h][4], q[h][5], q[h][6], q[h][7]);
+                rec[3 * f + 2] = make_float4(q[h][8], 0.f, 0.f, 0.f);
+                if (cdf_shared) {
+#pragma unroll
+                    for (int c = 0; c < S; ++c) remote(cdf, c)[f] = A[h];
+                } else {
+                    cdf[f] = A[h];
+                }
             }
         }
         if (bad) set_status(&s_err, DC_EINVAL);
@@ -432,6 +448,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
     // ---- points and keys: two points per thread and step, so that their chains of dependent
     // loads overlap ----
     const int i0 = (int)((long long)n * r / S), i1 = (int)((long long)n * (r + 1) / S);
+    float4* const xs = side ? w.y + base : w.x + base;
     bad = false;
     for (int ib = i0 + tid; ib < i1; ib += 2 * PREP_THREADS) {
         const int ii[2] = {ib, min(ib + PREP_THREADS, i1 - 1)};  // the last may be done twice
@@ -476,10 +493,8 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (!side) {
-                w.x[base + ii[h]] = x[h];
-                w.fw[base + ii[h]] = q[h];
-            }
+            xs[ii[h]] = x[h];
+            if (!side) w.fw[base + ii[h]] = q[h];
             w.tkey[gbase + ii[h]] = point_key(s_tab, box, x[h].x, x[h].y, x[h].z);
         }
     }
@@ -576,9 +591,9 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
     }
     meet();
 
-    // ---- (low key bits, index) and cell, in cell order; index bits: 32 - low >= those of n ----
-    unsigned* const ord = w.tord + gbase;
-    unsigned short* const cellof = w.tcell + gbase;
+    // ---- cell << 32 | low key bits | index, in cell order, in one store (stores to 32 lines
+    // take the load pipe 32 cycles whatever their width); index bits: 32 - low >= those of n ----
+    u64* const ord = w.tord + gbase;
     const int ibits = 32 - low;
     for (int ib = i0 + tid; ib < i1; ib += U * PREP_THREADS) {
         unsigned key[U];
@@ -593,8 +608,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
             if (i < i1) {
                 const int c = (int)(key[h] >> low);
                 const int pos = cell_add(hist, packed, c);
-                ord[pos] = (key[h] << ibits) | (unsigned)i;
-                cellof[pos] = (unsigned short)c;
+                ord[pos] = ((u64)c << 32) | ((key[h] << ibits) | (unsigned)i);
             }
         }
     }
@@ -603,34 +617,38 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
     // ---- rank within the cell, and the sorted points; the counters now hold the cells' ends,
     // the last slice's the ends over all slices ----
     {
-        const int* ends = remote(hist, S - 1);
+        if (S > 1) {  // a copy of them: the look-ups below stay in this CTA
+            if (r != S - 1)
+                for (int c = tid; c < words; c += PREP_THREADS) hist[c] = remote(hist, S - 1)[c];
+            __syncthreads();
+        }
+        const int* const ends = hist;
         static_assert(PREP_WARPS * REFINE_BUF * 4 <= REFINE_BYTES, "refine buffers");
         float* pts = w.tpts + 4 * gbase;
         const int p0 = (int)((long long)n * r / S), p1 = (int)((long long)n * (r + 1) / S);
         // per warp: the entries of its 32 positions' cells
         unsigned* buf = reinterpret_cast<unsigned*>(s_dyn) + CELL_BYTES / 4 + warp * REFINE_BUF;
+        u64 next = p0 + tid < p1 ? ord[p0 + tid] : 0ull;
         for (int pw = p0 + 32 * warp; pw < p1; pw += PREP_THREADS) {
             const int p = pw + lane;
             const bool on = p < p1;
-            const int pc = on ? p : p1 - 1;
-            const unsigned o = ord[pc];
-            const int cell = cellof[pc];
+            // beyond the last position: a copy of it
+            const int last = min(31, p1 - 1 - pw);
+            u64 cur = next;
+            if (last < 31) cur = __shfl_sync(0xffffffffu, cur, min(lane, last));
+            if (p + PREP_THREADS < p1) next = ord[p + PREP_THREADS];  // in flight meanwhile
+            const unsigned o = (unsigned)cur;
+            const int cell = (int)(cur >> 32);
             const int e = cell_get(ends, packed, cell);
             const int s = cell > 0 ? cell_get(ends, packed, cell - 1) : 0;
             const int i = (int)(o & ((1u << ibits) - 1u));
-            float x, y, z;
-            if (sampled) {
-                const float4 v = w.x[base + i];
-                x = v.x, y = v.y, z = v.z;
-            } else {
-                const float* v = (side ? fr.tgt : fr.pts) + 3LL * i;
-                x = v[0], y = v[1], z = v[2];
-            }
+            const float4 v = xs[i];
+            const float x = v.x, y = v.y, z = v.z;
             int pos = p;
             const int s0 = __shfl_sync(0xffffffffu, s, 0), e1 = __shfl_sync(0xffffffffu, e, 31);
             if (e1 - s0 <= REFINE_BUF) {  // the cells of consecutive positions are consecutive
                 __syncwarp();
-                for (int q = lane; q < e1 - s0; q += 32) buf[q] = ord[s0 + q];
+                for (int q = lane; q < e1 - s0; q += 32) buf[q] = (unsigned)ord[s0 + q];
                 __syncwarp();
                 pos = s;
 #pragma unroll 4
@@ -638,7 +656,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
             } else if (e - s <= REFINE_MAX) {
                 pos = s;
 #pragma unroll 4
-                for (int q = s; q < e; ++q) pos += ord[q] < o ? 1 : 0;
+                for (int q = s; q < e; ++q) pos += (unsigned)ord[q] < o ? 1 : 0;
             }
             if (!on) continue;
             float* b = pts + 32LL * (pos >> 3) + (pos & 7);
@@ -1114,16 +1132,43 @@ __global__ void __launch_bounds__(SINGLE_THREADS) k_tree_single(Ws w, int rows) 
         u64* slot = (side ? w.pba + fr->col0 : w.pab + fr->row0) + __float_as_int(__ldg(qb + 24));
         float R = __uint_as_float((unsigned)(*slot >> 32));  // the bound so far
         unsigned md = 0x7f800000u, mi = 0x7fffffffu;  // this lane's minimum and its index
+        // this lane's point of block b
+        auto point = [&](int b) {
+            const float* P = reinterpret_cast<const float*>(C.pts + 8LL * b) + sub;
+            const float dx = __fsub_rn(q.x, __ldg(P)), dy = __fsub_rn(q.y, __ldg(P + 8)),
+                        dz = __fsub_rn(q.z, __ldg(P + 16));
+            const unsigned i = __float_as_uint(__ldg(P + 24));
+            const unsigned db =
+                __float_as_uint(__fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx))));
+            if (db < md || (db == md && i < mi)) md = db, mi = i;
+        };
         for (int s = 0; s < C.nb2; s += 32) {
             const int i2 = s + lane;
-            bool hit = false;
+            float lb = INFINITY;
             if (i2 < C.nb2)
-                hit = box_bound(q, q, __ldg(C.box2 + 2 * i2), __ldg(C.box2 + 2 * i2 + 1)) <= R;
-            unsigned m2 = __ballot_sync(0xffffffffu, hit);
+                lb = box_bound(q, q, __ldg(C.box2 + 2 * i2), __ldg(C.box2 + 2 * i2 + 1));
+            unsigned m2 = __ballot_sync(0xffffffffu, i2 < C.nb2 && lb <= R);
+            if (s == 0 && __popc(m2) > 2) {
+                // a loose bound: the points of the nearest box of 64 in the nearest box of 512
+                const unsigned near2 = __reduce_min_sync(0xffffffffu, __float_as_uint(lb));
+                const int n2 = __ffs(__ballot_sync(0xffffffffu, __float_as_uint(lb) == near2)) - 1;
+                const int i1 = 8 * n2 + sub;
+                float l1 = INFINITY;
+                if (i1 < C.nb1)
+                    l1 = box_bound(q, q, __ldg(C.box1 + 2 * i1), __ldg(C.box1 + 2 * i1 + 1));
+                const unsigned near1 = __reduce_min_sync(0xffffffffu, __float_as_uint(l1));
+                const int n1 =
+                    8 * n2 + ((__ffs(__ballot_sync(0xffffffffu, __float_as_uint(l1) == near1)) - 1) & 7);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (8 * n1 + 4 * h + grp < C.nb) point(8 * n1 + 4 * h + grp);
+                R = fminf(R, __uint_as_float(__reduce_min_sync(0xffffffffu, md)));
+                m2 = __ballot_sync(0xffffffffu, i2 < C.nb2 && lb <= R);
+            }
             while (m2) {
                 const int t2 = take4(m2, grp);
                 const int i1 = (s + t2) * 8 + sub;
-                hit = false;
+                bool hit = false;
                 if (t2 >= 0 && i1 < C.nb1)
                     hit = box_bound(q, q, __ldg(C.box1 + 2 * i1), __ldg(C.box1 + 2 * i1 + 1)) <= R;
                 unsigned m1 = __ballot_sync(0xffffffffu, hit);
@@ -1137,15 +1182,7 @@ __global__ void __launch_bounds__(SINGLE_THREADS) k_tree_single(Ws w, int rows) 
                     while (m0) {
                         const int t0 = take4(m0, grp);
                         const int b = __shfl_sync(0xffffffffu, i0, t0 & 31);
-                        if (t0 >= 0) {
-                            const float* P = reinterpret_cast<const float*>(C.pts + 8LL * b) + sub;
-                            const float dx = __fsub_rn(q.x, __ldg(P)), dy = __fsub_rn(q.y, __ldg(P + 8)),
-                                        dz = __fsub_rn(q.z, __ldg(P + 16));
-                            const unsigned i = __float_as_uint(__ldg(P + 24));
-                            const unsigned db = __float_as_uint(
-                                __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx))));
-                            if (db < md || (db == md && i < mi)) md = db, mi = i;
-                        }
+                        if (t0 >= 0) point(b);
                     }
                     R = fminf(R, __uint_as_float(__reduce_min_sync(0xffffffffu, md)));
                 }
@@ -1213,7 +1250,7 @@ cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max
     e = launch_pdl(k_tree_search, total / SEARCH_THREADS, SEARCH_THREADS, 0, s, w, rows);
     count_launch();
     if (!e) {
-        e = launch_pdl(k_tree_single, std::min(8 * 152, total / SINGLE_THREADS), SINGLE_THREADS, 0,
+        e = launch_pdl(k_tree_single, std::min(16 * 152, total / SINGLE_THREADS), SINGLE_THREADS, 0,
                        s, w, rows);
         count_launch();
     }
