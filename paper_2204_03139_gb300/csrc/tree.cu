@@ -33,11 +33,11 @@ constexpr int KEY_BITS = 3 * KEY_AXIS_BITS;
 // 65 535 points, 2^14 cells with 32-bit counters), in 64 KB of shared memory at most
 constexpr int CELL_BITS_MIN = 10, CELL_BITS_PACKED = 15, CELL_BITS_WIDE = 14;
 constexpr int CELL_BYTES = 64 * 1024;
-constexpr int REFINE_BUF = 192;                     // entries a warp ranks from shared memory
-// a counting-sort cell of more points than this keeps them in arrival order (their rank by key
-// takes a comparison with every point of the cell)
-constexpr int REFINE_MAX = 512;
-constexpr int REFINE_BYTES = 12 * 1024;             // shared memory of all warps' buffers
+// a counting-sort cell of more points than this keeps them in arrival order (ranks are unique
+// within 256 consecutive positions, and the ranking window reaches that far to both sides)
+constexpr int REFINE_MAX = 256;
+constexpr int REFINE_RING = 4 * PREP_THREADS;       // entries of the ranking window's ring
+constexpr int REFINE_BYTES = REFINE_RING * 4;
 constexpr float PAD_COORD = 1e18f;                  // padding point of the last block of 8
 
 // ---------------------------------------------------------------------------------------
@@ -319,9 +319,8 @@ __device__ __forceinline__ int cell_get(const int* h, bool packed, int c) {
 //      points as given
 //   2. curve keys; histogram of their top bits (cells) in shared memory
 //   3. scan over cells and slices (through distributed shared memory), scatter of the points'
-//      (low key bits, index) and cell
-//   4. each point's rank within its cell by (key, index), which makes the order the same in
-//      every run; the sorted points as blocks of 8 (x[8] y[8] z[8] index[8], one 128-byte line)
+//      keys and indices
+//   4. each point's rank within its cell by its whole key; the sorted points as blocks of 8 (x[8] y[8] z[8] index[8], one 128-byte line)
 //   5. bounding boxes of 8, 64 and 512 consecutive points
 template <int S>
 __global__ void __launch_bounds__(PREP_THREADS, 2)
@@ -591,10 +590,9 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
     }
     meet();
 
-    // ---- cell << 32 | low key bits | index, in cell order, in one store (stores to 32 lines
-    // take the load pipe 32 cycles whatever their width); index bits: 32 - low >= those of n ----
+    // ---- index << 32 | key << 8, in cell order, in one store (stores to 32 lines take the load
+    // pipe 32 cycles whatever their width) ----
     u64* const ord = w.tord + gbase;
-    const int ibits = 32 - low;
     for (int ib = i0 + tid; ib < i1; ib += U * PREP_THREADS) {
         unsigned key[U];
 #pragma unroll
@@ -606,65 +604,79 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
         for (int h = 0; h < U; ++h) {
             const int i = ib + h * PREP_THREADS;
             if (i < i1) {
-                const int c = (int)(key[h] >> low);
-                const int pos = cell_add(hist, packed, c);
-                ord[pos] = ((u64)c << 32) | ((key[h] << ibits) | (unsigned)i);
+                const int pos = cell_add(hist, packed, (int)(key[h] >> low));
+                ord[pos] = ((u64)(unsigned)i << 32) | (key[h] << 8);
             }
         }
     }
     meet();
 
-    // ---- rank within the cell, and the sorted points; the counters now hold the cells' ends,
-    // the last slice's the ends over all slices ----
+    // ---- rank within the cell, and the sorted points. The counters now hold the cells' ends, the
+    // last slice's the ends over all slices. CTA r takes the r-th slice of the positions, one
+    // chunk of PREP_THREADS at a time; the keys of the chunks before and after stay in a ring in
+    // shared memory, so that a thread ranks its point among its cell's without waiting for
+    // memory, and the next chunk is in flight meanwhile. ----
     {
-        if (S > 1) {  // a copy of them: the look-ups below stay in this CTA
-            if (r != S - 1)
-                for (int c = tid; c < words; c += PREP_THREADS) hist[c] = remote(hist, S - 1)[c];
-            __syncthreads();
-        }
-        const int* const ends = hist;
-        static_assert(PREP_WARPS * REFINE_BUF * 4 <= REFINE_BYTES, "refine buffers");
-        float* pts = w.tpts + 4 * gbase;
         const int p0 = (int)((long long)n * r / S), p1 = (int)((long long)n * (r + 1) / S);
-        // per warp: the entries of its 32 positions' cells
-        unsigned* buf = reinterpret_cast<unsigned*>(s_dyn) + CELL_BYTES / 4 + warp * REFINE_BUF;
-        u64 next = p0 + tid < p1 ? ord[p0 + tid] : 0ull;
-        for (int pw = p0 + 32 * warp; pw < p1; pw += PREP_THREADS) {
-            const int p = pw + lane;
+        if (S > 1 && r != S - 1 && p0 < p1) {
+            // the ends of the cells that the slice meets
+            const int* last = remote(hist, S - 1);
+            const int ca = (int)((unsigned)ord[p0] >> (8 + low)) - 1;
+            const int cz = (int)((unsigned)ord[p1 - 1] >> (8 + low));
+            const int sh = packed ? 1 : 0;
+            for (int c = (max(ca, 0) >> sh) + tid; c <= cz >> sh; c += PREP_THREADS)
+                hist[c] = last[c];
+        }
+        unsigned* const ring = reinterpret_cast<unsigned*>(s_dyn) + CELL_BYTES / 4;
+        float* pts = w.tpts + 4 * gbase;
+        const int chunks = div_up(p1 - p0, PREP_THREADS);
+        auto fetch = [&](int c) {
+            const int p = p0 + c * PREP_THREADS + tid;
+            return p >= 0 && p < n ? ord[p] : ~0ull;
+        };
+        // keys with the position's low bits: all different among 256 consecutive positions
+        auto keep = [&](int c, u64 v) {
+            const int p = p0 + c * PREP_THREADS + tid;
+            ring[p & (REFINE_RING - 1)] = v == ~0ull ? ~0u : ((unsigned)v | (unsigned)(p & 255));
+        };
+        u64 cur = fetch(0), next = fetch(1), after = fetch(2);
+        keep(-1, fetch(-1));
+        keep(0, cur);
+        keep(1, next);
+        for (int ch = 0; ch < chunks; ++ch) {
+            __syncthreads();  // chunks ch - 1, ch and ch + 1 are in the ring
+            const int p = p0 + ch * PREP_THREADS + tid;
             const bool on = p < p1;
-            // beyond the last position: a copy of it
-            const int last = min(31, p1 - 1 - pw);
-            u64 cur = next;
-            if (last < 31) cur = __shfl_sync(0xffffffffu, cur, min(lane, last));
-            if (p + PREP_THREADS < p1) next = ord[p + PREP_THREADS];  // in flight meanwhile
-            const unsigned o = (unsigned)cur;
-            const int cell = (int)(cur >> 32);
-            const int e = cell_get(ends, packed, cell);
-            const int s = cell > 0 ? cell_get(ends, packed, cell - 1) : 0;
-            const int i = (int)(o & ((1u << ibits) - 1u));
+            const unsigned key = (unsigned)cur >> 8, o = (unsigned)cur | (unsigned)(p & 255);
+            const int i = (int)(cur >> 32);
+            keep(ch + 2, after);  // the slot of chunk ch - 2
+            cur = next;
+            next = after;
+            after = fetch(ch + 3);
+            if (!on) continue;
             const float4 v = xs[i];
             const float x = v.x, y = v.y, z = v.z;
+            const int cell = (int)(key >> low);
+            const int e = cell_get(hist, packed, cell);
+            const int s = cell > 0 ? cell_get(hist, packed, cell - 1) : 0;
             int pos = p;
-            const int s0 = __shfl_sync(0xffffffffu, s, 0), e1 = __shfl_sync(0xffffffffu, e, 31);
-            if (e1 - s0 <= REFINE_BUF) {  // the cells of consecutive positions are consecutive
-                __syncwarp();
-                for (int q = lane; q < e1 - s0; q += 32) buf[q] = (unsigned)ord[s0 + q];
-                __syncwarp();
-                pos = s;
-#pragma unroll 4
-                for (int q = s - s0; q < e - s0; ++q) pos += buf[q] < o ? 1 : 0;
-            } else if (e - s <= REFINE_MAX) {
-                pos = s;
-#pragma unroll 4
-                for (int q = s; q < e; ++q) pos += (unsigned)ord[q] < o ? 1 : 0;
+            if (e - s <= REFINE_MAX) {
+                // from a multiple of 4 on: the entries before s are of lower cells, those from e
+                // on of higher ones
+                pos = s & ~3;
+                for (int q = pos; q < e; q += 8) {
+                    const uint4 k0 = *reinterpret_cast<const uint4*>(ring + (q & (REFINE_RING - 1)));
+                    const uint4 k1 =
+                        *reinterpret_cast<const uint4*>(ring + ((q + 4) & (REFINE_RING - 1)));
+                    pos += (k0.x < o) + (k0.y < o) + (k0.z < o) + (k0.w < o) + (k1.x < o) +
+                           (k1.y < o) + (k1.z < o) + (k1.w < o);
+                }
             }
-            if (!on) continue;
             float* b = pts + 32LL * (pos >> 3) + (pos & 7);
             b[0] = x;
             b[8] = y;
             b[16] = z;
             b[24] = __int_as_float(i);
-            const unsigned key = ((unsigned)cell << low) | (o >> ibits);
             w.tkey[gbase + pos] = key;  // from here on in sorted order
             if ((pos & 7) == 0) w.tkb[gbase / 8 + (pos >> 3)] = key;
         }
