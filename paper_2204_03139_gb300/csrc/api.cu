@@ -88,6 +88,8 @@ Layout make_layout(const Sizes& s) {
     L.tbox1 = take(tp / 64 * 32);
     L.tbox2 = take(tp / TREE_STEP * 32);
     L.frec = take(s.tree ? s.sum_f * 48 : 0);
+    L.tgx = take(s.tree ? s.rows * 16 : 0);
+    L.grad4 = take(s.tree ? s.sum_v * 16 : 0);
     L.total = off;
     return L;
 }
@@ -134,6 +136,8 @@ Ws make_ws(void* base, const Layout& L) {
     w.tkb = reinterpret_cast<unsigned*>(p + L.tkb);
     w.tbox = reinterpret_cast<float4*>(p + L.tbox);
     w.tbox1 = reinterpret_cast<float4*>(p + L.tbox1);
+    w.tgx = reinterpret_cast<float4*>(p + L.tgx);
+    w.grad4 = reinterpret_cast<float4*>(p + L.grad4);
     w.frec = reinterpret_cast<float4*>(p + L.frec);
     w.tbox2 = reinterpret_cast<float4*>(p + L.tbox2);
     return w;
@@ -172,13 +176,17 @@ bool uniform_sizes(int T, int V, int F, int N, int M, Sizes& s, long long sub[3]
     s.n_frames = T;
     s.n_units = (long long)T * div_up(N, ROWS_PER_WARP);
     s.sum_f = (long long)T * F;
+    s.sum_v = (long long)T * V;
     s.rows = (long long)T * Npad;
     s.cols = (long long)T * Mpad;
     s.slices = epilogue_slices(T);
     // tensor-core regions, sized for both sides (the mode is not known here), when the frame
     // fits the key format; none for calls without targets
     s.tc_units = s.tc_slots = 0;
-    s.tree = with_tc && M > 0 && N <= TREE_MAX_POINTS && M <= TREE_MAX_POINTS ? 1 : 0;
+    s.tree = with_tc && M > 0 && N <= TREE_MAX_POINTS && M <= TREE_MAX_POINTS &&
+                     s.sum_v < INT_LIMIT
+                 ? 1
+                 : 0;
     if (with_tc && M > 0 && Npad <= TC_MAX_COLS && Mpad <= TC_MAX_COLS) {
         const long long u0 = div_up(N, TC_UNIT_ROWS), u1 = div_up(M, TC_UNIT_ROWS);
         s.tc_units = (long long)T * (u0 + u1);
@@ -234,6 +242,8 @@ int keyed_grid(int engine, long long chunks) {
     return engine == ENGINE_TC5 ? tc5_grid(chunks) : tc_grid(chunks);
 }
 
+constexpr int MAX_GRID_Y = 65535;
+
 int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total, void* ws,
                 size_t ws_bytes, cudaStream_t st, bool direct_only = false) {
     Sizes sz;
@@ -262,12 +272,17 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     // with sampling to follow, the tables and the area CDFs (and the frame boxes of the
     // tensor-core forms) share one launch
     const bool fused = (phases & PH_AREA) && (phases & PH_SAMPLE);
+    if (a.bwd && sz.tree && a.T <= MAX_GRID_Y) {
+        cudaError_t e = launch_backward(a, w, st);
+        return e ? cuda_fail(e, "kernel launch") : DC_OK;
+    }
     if (engine == ENGINE_TREE) {
         cudaError_t e = launch_tree(&a, w, T, a.pts ? 0 : a.F, std::max(a.N, a.M), rows, cols,
                                     a.mode, st);
-        if (!e && epi_flags)
-            e = launch_epilogue(w, T, a.slices, a.grad ? a.V : 0, a.mode, epi_flags, loss_total,
-                                1, st);
+        const int max_v = a.grad ? a.V : 0;
+        if (!e)
+            e = launch_tree_out(w, T, a.slices, epilogue_lanes(a.slices, max_v), max_v, rows, a.mode,
+                                loss_total, st);
         return e ? cuda_fail(e, "kernel launch") : DC_OK;
     }
     cudaError_t e = fused ? launch_build_area(a, w, st) : launch_build_uniform(a, w, st);
@@ -619,7 +634,7 @@ int dc_loss_traj_bwd(const float* verts, const int32_t* faces, const uint8_t* fa
 // batches
 // ---------------------------------------------------------------------------------------
 static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
-    s = Sizes{n, 0, 0, 0, 0, epilogue_slices(n), 0, 0, 1};
+    s = Sizes{n, 0, 0, 0, 0, epilogue_slices(n), 0, 0, 1, 0};
     sub[0] = sub[1] = sub[2] = 0;
     long long max_v = 0, tc_units = 0, tc_chunks = 0;
     bool tc_fits = true;
@@ -628,6 +643,7 @@ static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
         s.n_units += div_up(fr[k].N, ROWS_PER_WARP);
         for (int i = 0; i < 3; ++i) sub[i] += (long long)div_up(fr[k].N, ROWS_PER_WARP << i) * spu;
         s.sum_f += fr[k].F;
+        s.sum_v += fr[k].V;
         const long long Npad = (long long)div_up(fr[k].N, ROW_PAD) * ROW_PAD;
         const long long Mpad = (long long)div_up(fr[k].M, COL_PAD) * COL_PAD;
         s.rows += Npad;
@@ -639,6 +655,7 @@ static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
         tc_units += u0 + u1;
         tc_chunks += u0 * (Mpad / TC_CHUNK) + u1 * (Npad / TC_CHUNK);
     }
+    if (s.sum_v >= INT_LIMIT) s.tree = 0;
     if (tc_fits && tc_chunks < INT_LIMIT) {
         s.tc_units = tc_units;
         s.tc_slots = tc_grid(tc_chunks);
@@ -743,7 +760,7 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
     int* turb = reinterpret_cast<int*>(tcimg.data() + (L.tc_urb - tc_beg));
     int* tupre = reinterpret_cast<int*>(tcimg.data() + (L.tc_upre - tc_beg));
     int tunit = 0, tchunk = 0;
-    int row0 = 0, col0 = 0, cdf0 = 0, unit = 0, subc = 0, any_grad = 0, max_v = 0, max_f = 0, max_n = 0;
+    int row0 = 0, col0 = 0, cdf0 = 0, v0 = 0, unit = 0, subc = 0, any_grad = 0, max_v = 0, max_f = 0, max_n = 0;
     // The table lists the frames largest first (N + M, ties in the caller's order). The
     // sampling and epilogue kernels run one CTA per (frame, slice) in table order, so the
     // long CTAs of big frames start first and the small ones fill in behind them instead of
@@ -764,8 +781,9 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
         d.loss = f.loss ? f.loss : w.loss + k;
         d.Npad = div_up(f.N, ROW_PAD) * ROW_PAD;
         d.Mpad = div_up(f.M, COL_PAD) * COL_PAD;
-        d.nn_ab = f.nn_ab ? f.nn_ab : w.nnab + row0;
-        d.nn_ba = f.nn_ba ? f.nn_ba : w.nnba + col0;
+        const bool tree = engine == ENGINE_TREE;  // needs no neighbour buffers of its own
+        d.nn_ab = f.nn_ab || tree ? f.nn_ab : w.nnab + row0;
+        d.nn_ba = f.nn_ba || tree ? f.nn_ba : w.nnba + col0;
         d.grad = f.grad_verts;
         d.V = f.V;
         d.F = f.F;
@@ -777,6 +795,7 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
         d.row0 = row0;
         d.col0 = col0;
         d.cdf0 = cdf0;
+        d.v0 = v0;
         d.unit0 = unit;
         d.tc_unit0 = tunit;
         fd[k] = d;
@@ -811,6 +830,7 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
         row0 += d.Npad;
         col0 += d.Mpad;
         cdf0 += f.F;
+        v0 += f.V;
     }
     rowpre[n_frames] = row0;
     colpre[n_frames] = col0;
@@ -887,10 +907,10 @@ int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream) {
     if (p.engine == ENGINE_TREE && stall_pending()) p.engine = ENGINE_DIRECT;
     if (p.engine == ENGINE_TREE) {
         cudaError_t e = launch_tree(nullptr, w, n, p.max_f, p.max_n, rows, cols, p.mode, stream);
+        const int max_v = p.any_grad ? p.max_v : 0, slices = (int)p.sz.slices;
         if (!e)
-            e = launch_epilogue(w, n, (int)p.sz.slices, p.any_grad ? p.max_v : 0, p.mode,
-                                EPI_RESCAN | EPI_LOSS | (p.any_grad ? EPI_GRAD : 0), loss_total,
-                                1, stream);
+            e = launch_tree_out(w, n, slices, epilogue_lanes(slices, max_v), max_v, rows, p.mode,
+                                loss_total, stream);
         return e ? cuda_fail(e, "dc_batch_run") : DC_OK;
     }
     const bool tc = keyed(p.engine);

@@ -164,6 +164,7 @@ struct FrameDesc {
     int row0;             // offset of this frame's sim points in the padded row buffers
     int col0;             // offset of this frame's targets in the padded column buffers
     int cdf0;             // offset of this frame's CDF
+    int v0;               // offset of this frame's vertices in the gradient accumulators
     int unit0;            // first Chamfer unit of this frame
     int skip;             // weight (or gradient multiplier) 0: no work, L reported as 0
     int tc_unit0;         // first tensor-core unit of this frame (sim rows, then targets)
@@ -197,7 +198,7 @@ struct WsHeader {
 struct Layout {
     size_t hdr, frames, rowpre, colpre, unit_frame, unit_rb, unit_pre, cdf, x, fw, tsoa, tpl,
         pab, pba, nnab, nnba, loss, part, frame_err, fbox, tc_ufr, tc_urb, tc_upre, tca, tcb,
-        kab, kba, kpart, tcfb, tcfn, step_frame, y, tkey, tord, tpts, tkb, tbox, tbox1, tbox2, frec, total;
+        kab, kba, kpart, tcfb, tcfn, step_frame, y, tkey, tord, tpts, tkb, tbox, tbox1, tbox2, frec, tgx, grad4, total;
 };
 
 struct Sizes {
@@ -206,6 +207,7 @@ struct Sizes {
     long long tc_units;  // tensor-core units (0: no tensor-core regions)
     long long tc_slots;  // CTAs the partial-key buffer is sized for
     long long tree;      // 1: regions of the pruned search
+    long long sum_v;     // vertices of all frames
 };
 
 // Epilogue slices per frame: as many as keep all (frame, slice) CTAs in one wave, at most
@@ -262,6 +264,8 @@ struct Ws {
     unsigned* tkb;             // [(rows + cols) / 8] first key of every block
     float4* tbox;              // [(rows + cols) / 8][2] (lo, hi) of 8 points
     float4* tbox1;             // [(rows + cols) / 64][2] of 64
+    float4* tgx;               // [rows] gradient of the sim points, sorted order
+    float4* grad4;             // [sum V] gradient of the vertices, 16 bytes each
     float4* frec;              // [sum F][3] corners of every face, per frame (sampled frames)
     float4* tbox2;             // [(rows + cols) / TREE_STEP][2] of 512 (from the frame's start)
 };
@@ -381,6 +385,17 @@ int tuned_warps();
 enum : int { EPI_RESCAN = 1, EPI_LOSS = 2, EPI_GRAD = 4 };
 cudaError_t launch_epilogue(const Ws& w, int n_frames, int slices, int max_v, int mode,
                             int flags, float* total, int exact, cudaStream_t s);
+cudaError_t launch_frame_loss(const Ws& w, int n_frames, int slices, int bidir, float* total,
+                              cudaStream_t s);
+// rows that the epilogue's CTA sums side by side (the order of its loss partials)
+int epilogue_lanes(int slices, int max_v);
+// losses, neighbours and gradients after launch_tree
+cudaError_t launch_tree_out(const Ws& w, int n_frames, int slices, int lanes, int max_v, int rows,
+                            int mode, float* total, cudaStream_t s);
+// vertex gradients from their accumulators to the caller's arrays
+cudaError_t launch_grad_out(const Ws& w, int n_frames, int max_v, cudaStream_t s);
+// the recomputing backward of a uniform trajectory (needs the pruned search's regions)
+cudaError_t launch_backward(const UniformArgs& a, const Ws& w, cudaStream_t s);
 // sum_t w_t L_t of given per-frame losses, in the fixed order of the trajectory calls
 cudaError_t launch_loss_total(const float* lf, const float* w, int T, float* total,
                               cudaStream_t s);

@@ -37,8 +37,12 @@ __device__ __forceinline__ FrameDesc uniform_frame(const UniformArgs& a, const W
     f.pts = a.pts ? a.pts + 3LL * k * a.N : nullptr;
     f.tgt = a.tgt ? a.tgt + 3LL * k * a.M : nullptr;
     f.loss = a.loss ? a.loss + k : w.loss + k;
-    f.nn_ab = a.nn_ab ? a.nn_ab + (long long)k * a.N : w.nnab + (long long)k * Npad;
-    f.nn_ba = a.nn_ba ? a.nn_ba + (long long)k * a.M : w.nnba + (long long)k * Mpad;
+    // the pruned search needs no neighbour buffers of its own
+    const bool tree = a.engine == ENGINE_TREE;
+    f.nn_ab = a.nn_ab ? a.nn_ab + (long long)k * a.N
+                      : (tree ? nullptr : w.nnab + (long long)k * Npad);
+    f.nn_ba = a.nn_ba ? a.nn_ba + (long long)k * a.M
+                      : (tree ? nullptr : w.nnba + (long long)k * Mpad);
     f.grad = a.grad ? a.grad + 3LL * k * a.V : nullptr;
     f.out_pts = a.out_pts ? a.out_pts + 3LL * k * a.N : nullptr;
     f.out_face = a.out_face ? a.out_face + (long long)k * a.N : nullptr;
@@ -54,6 +58,7 @@ __device__ __forceinline__ FrameDesc uniform_frame(const UniformArgs& a, const W
     f.row0 = k * Npad;
     f.col0 = k * Mpad;
     f.cdf0 = k * a.F;
+    f.v0 = k * a.V;
     f.unit0 = 0;
     f.tc_unit0 = 0;
     return f;
@@ -160,6 +165,24 @@ __device__ __forceinline__ int pick_face(const float* cdf, int F, float rf) {
     return min(lo, F - 1);
 }
 
+// pick_face of two draws at once: their binary searches' dependent loads overlap
+__device__ __forceinline__ void pick_face2(const float* cdf, int F, float ra, float rb, int& fa,
+                                           int& fb) {
+    const float A = cdf[F - 1];
+    const float ta = __fmul_rn(ra, A), tb = __fmul_rn(rb, A);
+    int la = 0, lb = 0;  // first f with cdf[f] > t, by halving steps over [l, l + len)
+    for (int len = F; len > 0;) {
+        const int half = len >> 1;
+        const bool ga = cdf[min(la + half, F - 1)] <= ta && la + half < F;
+        const bool gb = cdf[min(lb + half, F - 1)] <= tb && lb + half < F;
+        la = ga ? la + half + 1 : la;
+        lb = gb ? lb + half + 1 : lb;
+        len = half;
+    }
+    fa = min(la, F - 1);
+    fb = min(lb, F - 1);
+}
+
 // barycentric weights of the draw (r1, r2), and the point's coordinate with corners a, b, c
 __device__ __forceinline__ void bary_weights(float r1, float r2, float& w0, float& w1, float& w2) {
     const float s = __fsqrt_rn(r1);
@@ -195,6 +218,37 @@ __device__ __forceinline__ bool pick_point(const float* cdf, int F, int V,
     x.z = bary_point(w0, w1, w2, p0[2], p1[2], p2[2]);
     q = make_int4(f, __float_as_int(w0), __float_as_int(w1), __float_as_int(w2));
     return true;
+}
+
+// ---- gradient accumulators of 16 bytes ----
+__device__ __forceinline__ void red_add4(float4* p, float x, float y, float z) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z),
+                 "f"(0.0f)
+                 : "memory");
+}
+
+// Multiplier of (point - neighbour) in dL/dpoint for the queries of a side: 2 g / N (sim points)
+// or 2 g / M (targets) in Eq. 1, 2 g in Eq. 2 (the derivative of the squared distance); 0 when
+// the frame has no gradient.
+__device__ __forceinline__ float grad_scale(const FrameDesc* fr, int side, int bidir) {
+    if (!fr->grad || !fr->verts) return 0.0f;
+    const float g = __fmul_rn(2.0f, fr->gscale);
+    return bidir ? __fdiv_rn(g, (float)(side ? fr->M : fr->N)) : g;
+}
+
+
+// a sim point's gradient g to the vertices of its face (q: face, weights) of frame fr
+__device__ __forceinline__ void scatter_face(const Ws& w, const FrameDesc* fr, int4 q, float4 g) {
+    const float wt[3] = {__int_as_float(q.y), __int_as_float(q.z), __int_as_float(q.w)};
+    const int* f = fr->faces + 3LL * q.x;
+    int v[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = __ldg(f + k);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        if ((unsigned)v[k] < (unsigned)fr->V)
+            red_add4(w.grad4 + fr->v0 + v[k], __fmul_rn(wt[k], g.x), __fmul_rn(wt[k], g.y),
+                     __fmul_rn(wt[k], g.z));
 }
 
 }  // namespace

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
                         kahan_add(sab, cab_c, __uint_as_float((unsigned)(pr[r] >> 32)));
                     if (pr[r] == EMPTY || (unsigned)nn >= (unsigned)M)
                         set_status(&w.hdr->status, DC_EDEVICE);
-                    fr->nn_ab[ir[r]] = nn;
+                    if (fr->nn_ab) fr->nn_ab[ir[r]] = nn;
                 }
                 nr[r] = vr[r] && (unsigned)nn < (unsigned)M && q < 3 ? nn : -1;
             }
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
             if (valid && q == 0) {
                 if (p != EMPTY && want_loss) kahan_add(sab, cab_c, dmin);
                 if (nn < 0) set_status(&w.hdr->status, DC_EDEVICE);
-                fr->nn_ab[i] = nn;
+                if (fr->nn_ab) fr->nn_ab[i] = nn;
             }
         } else if (valid) {
             nn = fr->nn_ab[i];
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
                             kahan_add(sba, cba_c, __uint_as_float((unsigned)(pr[r] >> 32)));
                         if (pr[r] == EMPTY || (unsigned)nn >= (unsigned)N)
                             set_status(&w.hdr->status, DC_EDEVICE);
-                        fr->nn_ba[jr[r]] = nn;
+                        if (fr->nn_ba) fr->nn_ba[jr[r]] = nn;
                     }
                     nr[r] = vr[r] && (unsigned)nn < (unsigned)N && q < 3 ? nn : -1;
                 }
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
                 if (valid && q == 0) {
                     if (p != EMPTY && want_loss) kahan_add(sba, cba_c, dmin);
                     if (nn < 0) set_status(&w.hdr->status, DC_EDEVICE);
-                    fr->nn_ba[j] = nn;
+                    if (fr->nn_ba) fr->nn_ba[j] = nn;
                 }
             } else if (valid) {
                 nn = fr->nn_ba[j];
@@ -509,12 +509,24 @@ cudaError_t launch_epilogue(const Ws& w, int n_frames, int slices, int max_v, in
                                : launch_pdl(k_epilogue<EPI_THREADS>, n_frames * slices,
                                             EPI_THREADS, 0, s, w, a);
     count_launch();
-    if (!e && (flags & EPI_LOSS)) {
-        e = launch_pdl(k_frame_loss, 1, LOSS_THREADS, 0, s, w, n_frames, slices, (int)a.bidir,
-                       total);
-        count_launch();
-    }
+    if (!e && (flags & EPI_LOSS)) e = launch_frame_loss(w, n_frames, slices, a.bidir, total, s);
     return e ? e : cudaGetLastError();
+}
+
+cudaError_t launch_frame_loss(const Ws& w, int n_frames, int slices, int bidir, float* total,
+                              cudaStream_t s) {
+    cudaError_t e =
+        launch_pdl(k_frame_loss, 1, LOSS_THREADS, 0, s, w, n_frames, slices, bidir, total);
+    count_launch();
+    return e ? e : cudaGetLastError();
+}
+
+int epilogue_lanes(int slices, int max_v) {
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const bool one = slices == 1 && max_v > 0 && (size_t)max_v * 12 + 1024 <= (size_t)optin;
+    return (one ? EPI_THREADS_ONE_SLICE : EPI_THREADS) / 4;
 }
 
 cudaError_t launch_loss_total(const float* lf, const float* w, int T, float* total,

@@ -276,24 +276,6 @@ __device__ __forceinline__ void face_record2(const float* __restrict__ verts,
     }
 }
 
-// pick_face of two draws at once: their binary searches' dependent loads overlap
-__device__ __forceinline__ void pick_face2(const float* cdf, int F, float ra, float rb, int& fa,
-                                           int& fb) {
-    const float A = cdf[F - 1];
-    const float ta = __fmul_rn(ra, A), tb = __fmul_rn(rb, A);
-    int la = 0, lb = 0;  // first f with cdf[f] > t, by halving steps over [l, l + len)
-    for (int len = F; len > 0;) {
-        const int half = len >> 1;
-        const bool ga = cdf[min(la + half, F - 1)] <= ta && la + half < F;
-        const bool gb = cdf[min(lb + half, F - 1)] <= tb && lb + half < F;
-        la = ga ? la + half + 1 : la;
-        lb = gb ? lb + half + 1 : lb;
-        len = half;
-    }
-    fa = min(la, F - 1);
-    fb = min(lb, F - 1);
-}
-
 // Counting-sort cells of n points: 2^bits of them
 __device__ __forceinline__ int cell_bits(int n, int most) {
     int b = CELL_BITS_MIN;
@@ -392,9 +374,10 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
     // the steps of the search (TREE_STEP queries each) find their frame here
     for (int s = r * PREP_THREADS + tid; s < npad / TREE_STEP; s += S * PREP_THREADS)
         w.step_frame[gbase / TREE_STEP + s] = k;
-    if (side == 0 && fr.grad)
-        for (int e = r * PREP_THREADS + tid; e < 3 * fr.V; e += S * PREP_THREADS)
-            fr.grad[e] = 0.0f;
+    const bool grad = side == 0 && fr.grad && fr.verts;  // its accumulators start from zero
+    if (grad)
+        for (int v = r * PREP_THREADS + tid; v < fr.V; v += S * PREP_THREADS)
+            w.grad4[fr.v0 + v] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (fr.skip) {  // the same for the whole cluster
         if (tid == 0 && r == 0) w.frame_err[2 * k + side] = DC_OK;
         pdl_trigger();
@@ -494,6 +477,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
         for (int h = 0; h < 2; ++h) {
             xs[ii[h]] = x[h];
             if (!side) w.fw[base + ii[h]] = q[h];
+            if (grad) w.tgx[base + ii[h]] = make_float4(0.f, 0.f, 0.f, 0.f);
             w.tkey[gbase + ii[h]] = point_key(s_tab, box, x[h].x, x[h].y, x[h].z);
         }
     }
@@ -891,7 +875,7 @@ __device__ __forceinline__ TreeCols tree_cols(const Ws& w, const FrameDesc* fr, 
 //     queries of a tile that meets too many boxes, and queries that met their minimum in two
 //     blocks (exact ties, whose lowest index must win) are queued for k_tree_single.
 __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
-    k_tree_search(Ws w, int rows) {
+    k_tree_search(Ws w, int rows, int bidir) {
     pdl_wait();
     __shared__ TreeWarp s_warp[SEARCH_THREADS / 32];
     const int lane = threadIdx.x & 31, t = lane & 3, g = lane >> 2;
@@ -1082,31 +1066,52 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
         }
     }
 
-    // the indices: the lowest one attaining the query's minimum among the quad's lanes
+    // The indices: the lowest one attaining the query's minimum among the quad's lanes, and its
+    // place in the sorted order; lane t keeps those of the quad's t-th query, its own.
     float md = own;
-    int nn = 0x7fffffff;
+    int nn = 0x7fffffff, at = 0;
     bool alone = valid && (wide || !act);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         float v = best[j];
         v = fminf(v, __shfl_xor_sync(0xffffffffu, v, 1));
         v = fminf(v, __shfl_xor_sync(0xffffffffu, v, 2));
-        int i = 0x7fffffff;
+        int i = 0x7fffffff, p = 8 * bblk[j] + 2 * t;
         if (bblk[j] >= 0 && best[j] == v) {
             const float2* P = reinterpret_cast<const float2*>(C.pts + 8LL * bblk[j]) + t;
             const float2 d = dist2x2(__ldg(P), __ldg(P + 4), __ldg(P + 8), nx[j], ny[j], nz[j]);
             const float2 id = __ldg(P + 12);
             if (d.x == v) i = __float_as_int(id.x);
-            if (d.y == v) i = min(i, __float_as_int(id.y));
+            if (d.y == v && __float_as_int(id.y) < i) {
+                i = __float_as_int(id.y);
+                ++p;
+            }
         }
+        const int mine = i;
         i = min(i, __shfl_xor_sync(0xffffffffu, i, 1));
         i = min(i, __shfl_xor_sync(0xffffffffu, i, 2));
+        // indices are distinct: one lane holds the minimum
+        const unsigned holds = __ballot_sync(0xffffffffu, mine == i) >> (lane & ~3);
+        p = __shfl_sync(0xffffffffu, p, (lane & ~3) + ((__ffs(holds) - 1) & 3));
         const unsigned tm = __ballot_sync(0xffffffffu, tie[j] && best[j] == v);
         if (t == j) {
             alone = alone || (valid && ((tm >> (lane & ~3)) & 0xfu) != 0);
             nn = i;
+            at = p;
             md = fminf(md, v);
         }
+    }
+    // the pair's gradient, added to the sim point's (the query's own, or its neighbour's for a
+    // target query), 16 bytes at once
+    const float gs = grad_scale(fr, side, bidir);
+    if (gs != 0.0f && valid && !alone && nn != 0x7fffffff) {
+        const float* A = w.tpts + 4LL * (gt - pos0) + 32LL * ((pos0 + lane) >> 3) + ((pos0 + lane) & 7);
+        const float* B = reinterpret_cast<const float*>(C.pts) + 32LL * (at >> 3) + (at & 7);
+        const float sg = side ? -gs : gs;  // sim point - target, whichever is the query
+        red_add4(w.tgx + fr->row0 + (side ? at : pos0 + lane),
+                 __fmul_rn(sg, __fsub_rn(__ldg(A), __ldg(B))),
+                 __fmul_rn(sg, __fsub_rn(__ldg(A + 8), __ldg(B + 8))),
+                 __fmul_rn(sg, __fsub_rn(__ldg(A + 16), __ldg(B + 16))));
     }
     if (valid) {
         // this lane's query's index; the slot of a queued query carries its bound
@@ -1128,7 +1133,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
 // The queued queries, one warp each: the same walk with the query's own box (a point), every
 // lane one point of four blocks of 8.
 constexpr int SINGLE_THREADS = 128;
-__global__ void __launch_bounds__(SINGLE_THREADS) k_tree_single(Ws w, int rows) {
+__global__ void __launch_bounds__(SINGLE_THREADS, 16) k_tree_single(Ws w, int rows, int bidir) {
     pdl_wait();
     const int lane = threadIdx.x & 31, grp = lane >> 3, sub = lane & 7;
     const int count = w.hdr->tree_n;
@@ -1144,6 +1149,7 @@ __global__ void __launch_bounds__(SINGLE_THREADS) k_tree_single(Ws w, int rows) 
         u64* slot = (side ? w.pba + fr->col0 : w.pab + fr->row0) + __float_as_int(__ldg(qb + 24));
         float R = __uint_as_float((unsigned)(*slot >> 32));  // the bound so far
         unsigned md = 0x7f800000u, mi = 0x7fffffffu;  // this lane's minimum and its index
+        int mb = 0;                                    // and its block
         // this lane's point of block b
         auto point = [&](int b) {
             const float* P = reinterpret_cast<const float*>(C.pts + 8LL * b) + sub;
@@ -1152,7 +1158,7 @@ __global__ void __launch_bounds__(SINGLE_THREADS) k_tree_single(Ws w, int rows) 
             const unsigned i = __float_as_uint(__ldg(P + 24));
             const unsigned db =
                 __float_as_uint(__fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx))));
-            if (db < md || (db == md && i < mi)) md = db, mi = i;
+            if (db < md || (db == md && i < mi)) md = db, mi = i, mb = b;
         };
         for (int s = 0; s < C.nb2; s += 32) {
             const int i2 = s + lane;
@@ -1203,8 +1209,100 @@ __global__ void __launch_bounds__(SINGLE_THREADS) k_tree_single(Ws w, int rows) 
         const unsigned dm = __reduce_min_sync(0xffffffffu, md);
         const unsigned im = __reduce_min_sync(0xffffffffu, md == dm ? mi : 0x7fffffffu);
         if (lane == 0) *slot = im == 0x7fffffffu ? EMPTY : ((u64)dm << 32) | im;
+        const float gs = grad_scale(fr, side, bidir);
+        const unsigned who = __ballot_sync(0xffffffffu, md == dm && mi == im);
+        if (gs != 0.0f && im != 0x7fffffffu && lane == __ffs(who) - 1) {
+            const float* P = reinterpret_cast<const float*>(C.pts + 8LL * mb) + sub;
+            const float sg = side ? -gs : gs;
+            red_add4(w.tgx + fr->row0 + (side ? 8 * mb + sub : pos),
+                     __fmul_rn(sg, __fsub_rn(q.x, __ldg(P))),
+                     __fmul_rn(sg, __fsub_rn(q.y, __ldg(P + 8))),
+                     __fmul_rn(sg, __fsub_rn(q.z, __ldg(P + 16))));
+        }
     }
     pdl_trigger();
+}
+
+// ---------------------------------------------------------------------------------------
+// losses and vertex gradients
+// ---------------------------------------------------------------------------------------
+constexpr int OUT_THREADS = 256;
+
+// Blocks [0, loss_blocks): the loss partials of OUT_THREADS / lanes (frame, slice)s each, and the
+// neighbours where the caller wants them, from the (distance, index) records, coalesced. `lanes`
+// threads sum a slice in the order of the general epilogue (a thread per row, every lanes-th row;
+// then a tree over the threads), so the losses are bit for bit those of the other engines.
+// The other blocks: TREE_STEP sim points in sorted order each, their gradient spread over their
+// face's vertices with the barycentric weights (Eq. 4), 16 bytes per vertex. In sorted order
+// neighbouring points share faces and vertices, so the face look-ups hit L1; against one atomic
+// per coordinate and (point, target) pair the points' sums save half the scatter, and vectors
+// two thirds of the rest (64 uneven trajectories: 3.8 ms as one epilogue, 1.5 ms here).
+__global__ void __launch_bounds__(OUT_THREADS) k_tree_out(Ws w, int n_frames, int slices, int lanes,
+                                                          int loss_blocks, int bidir) {
+    pdl_entry();
+    const int tid = threadIdx.x;
+    if ((int)blockIdx.x >= loss_blocks) {
+        const int step = blockIdx.x - loss_blocks;
+        const FrameDesc* fr = w.frames + w.step_frame[step];
+        if (fr->skip || !fr->grad || !fr->verts) return;
+        const int g = step * TREE_STEP + tid, p = g - fr->row0;
+        if (p >= fr->N) return;
+        const float4 gr = w.tgx[g];
+        const int i = __float_as_int(__ldg(w.tpts + 4LL * fr->row0 + 32LL * (p >> 3) + 24 + (p & 7)));
+        const int4 q = __ldg(w.fw + fr->row0 + i);
+        if (q.x < 0) return;
+        scatter_face(w, fr, q, gr);
+        return;
+    }
+    __shared__ float s_red[2][OUT_THREADS / 8];
+    const int ks = blockIdx.x * (OUT_THREADS / lanes) + tid / lanes, t = tid & (lanes - 1);
+    const bool on = ks < n_frames * slices;
+    const int k = on ? ks / slices : 0, sl = on ? ks - k * slices : 0;
+    const FrameDesc* fr = w.frames + k;
+    const bool live = on && !fr->skip;
+#pragma unroll 1
+    for (int side = 0; side < (bidir ? 2 : 1); ++side) {
+        const int n = side ? fr->M : fr->N, nc = side ? fr->N : fr->M;
+        const u64* rec = side ? w.pba + fr->col0 : w.pab + fr->row0;
+        int* nn = side ? fr->nn_ba : fr->nn_ab;
+        const int a = (int)((long long)n * sl / slices), b = (int)((long long)n * (sl + 1) / slices);
+        float s = 0.f, c = 0.f;
+        bool bad = false;
+        if (live) {
+#pragma unroll 4
+            for (int i = a + t; i < b; i += lanes) {
+                const u64 p = __ldg(rec + i);
+                const unsigned j = (unsigned)p;
+                if (p != EMPTY) {  // compensated sum
+                    const float y = __fsub_rn(__uint_as_float((unsigned)(p >> 32)), c);
+                    const float u = __fadd_rn(s, y);
+                    c = __fsub_rn(__fsub_rn(u, s), y);
+                    s = u;
+                }
+                bad |= p == EMPTY || j >= (unsigned)nc;
+                if (nn) nn[i] = p == EMPTY ? -1 : (int)j;
+            }
+        }
+        if (bad) set_status(&w.hdr->status, DC_EDEVICE);
+        // eight threads at a time, then over their sums
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s = __fadd_rn(s, __shfl_down_sync(0xffffffffu, s, o, 8));
+        if ((tid & 7) == 0) s_red[side][tid >> 3] = s;
+    }
+    __syncthreads();
+    // one thread per side of each slice; the tree of a warp over lanes / 8 values, zeros beyond
+    const int sides = tid & 1, q = tid >> 1, at = blockIdx.x * (OUT_THREADS / lanes) + q;
+    if (q < OUT_THREADS / lanes && at < n_frames * slices) {
+        float v[OUT_THREADS / 8];
+#pragma unroll
+        for (int i = 0; i < OUT_THREADS / 8; ++i)
+            v[i] = i < lanes / 8 && (sides == 0 || bidir) ? s_red[sides][q * (lanes / 8) + i] : 0.f;
+#pragma unroll
+        for (int o = OUT_THREADS / 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < o; ++i) v[i] = __fadd_rn(v[i], v[i + o]);
+        w.part[2 * at + sides] = v[0];
+    }
 }
 
 int g_prep_smem[64];  // per device: dynamic shared memory the preparation may use
@@ -1259,15 +1357,29 @@ cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max
     if (e) return e;
     prof_before(s);
     const int total = rows + (mode == DC_BIDIR_MEAN ? cols : 0);
-    e = launch_pdl(k_tree_search, total / SEARCH_THREADS, SEARCH_THREADS, 0, s, w, rows);
+    const int bidir = mode == DC_BIDIR_MEAN;
+    e = launch_pdl(k_tree_search, total / SEARCH_THREADS, SEARCH_THREADS, 0, s, w, rows, bidir);
     count_launch();
     if (!e) {
         e = launch_pdl(k_tree_single, std::min(16 * 152, total / SINGLE_THREADS), SINGLE_THREADS, 0,
-                       s, w, rows);
+                       s, w, rows, bidir);
         count_launch();
     }
     prof_after(s);
     return e ? e : cudaGetLastError();
+}
+
+// After launch_tree: loss partials, neighbours, gradients, then the frame losses and their total.
+// max_v: largest V of the frames with a gradient (0: no gradient).
+cudaError_t launch_tree_out(const Ws& w, int n_frames, int slices, int lanes, int max_v, int rows,
+                            int mode, float* total, cudaStream_t s) {
+    const int bidir = mode == DC_BIDIR_MEAN;
+    const int loss_blocks = div_up(n_frames * slices, OUT_THREADS / lanes);
+    cudaError_t e = launch_pdl(k_tree_out, loss_blocks + (max_v > 0 ? rows / TREE_STEP : 0),
+                               OUT_THREADS, 0, s, w, n_frames, slices, lanes, loss_blocks, bidir);
+    count_launch();
+    if (!e && max_v > 0) e = launch_grad_out(w, n_frames, max_v, s);
+    return e ? e : launch_frame_loss(w, n_frames, slices, bidir, total, s);
 }
 
 }  // namespace dc
