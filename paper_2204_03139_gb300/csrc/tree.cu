@@ -15,6 +15,8 @@
 // per 32 consecutive queries of the sorted order.
 #include <cooperative_groups.h>
 
+#include <cfloat>
+
 #include <algorithm>
 
 #include "dc_sampling.cuh"
@@ -698,6 +700,8 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
                             hi[c] = fmaxf(hi[c], t[j]);
                         }
                 }
+            }
+            if (b < (nb + 7) / 8 * 8) {  // empty boxes up to a whole box of 64
                 box0[2 * b] = make_float4(lo[0], lo[1], lo[2], 0.f);
                 box0[2 * b + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
             }
@@ -748,7 +752,10 @@ constexpr int WIDE_BOX2 = 16;
 constexpr int WIDE_BOX1 = 40;
 // Boxes of 64 points on their way to a warp: their eight boxes of 8 and their points are copied
 // to shared memory while the ones before are searched.
-constexpr int STAGES = 3;
+#ifndef DC_TREE_STAGES
+#define DC_TREE_STAGES 2
+#endif
+constexpr int STAGES = DC_TREE_STAGES;  // a power of two
 struct TreeStage {
     float4 pts[64];  // eight blocks of x[8] y[8] z[8] index[8]
     float4 box[16];  // (lo, hi) of the eight blocks
@@ -943,23 +950,23 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
         block_dist(C.pts + 8LL * lo, make_float2(-qx, -qx), make_float2(-qy, -qy),
                    make_float2(-qz, -qz), d);
         const float m = block_min(d);
-        own = m <= INFINITY ? m : INFINITY;  // NaN: no bound
+        own = m <= FLT_MAX ? m : FLT_MAX;  // NaN: no bound (empty boxes, at infinity, stay out)
         // outliers: a bound 2^OUTLIER_LOG2 or more above the others' (mean of the exponents)
-        const int e = (int)(__float_as_uint(own) >> 23);
-        const int mean = __reduce_add_sync(0xffffffffu, valid ? e : 0) / min(32, n - pos0);
-        act = valid && (e <= mean + OUTLIER_LOG2 || own == INFINITY);
+        const int e = (int)(__float_as_uint(own) >> 23), count = min(32, n - pos0);
+        const int sum = __reduce_add_sync(0xffffffffu, valid ? e : 0);
+        act = valid && (e * count <= sum + OUTLIER_LOG2 * count || own == FLT_MAX);
     }
     // per query of the quad: the bound (-1: not searched here), the same in all four lanes; this
-    // lane's minimum and its block, and whether the minimum was met in another block too
+    // lane's minimum, the blocks it was met in (box of 64 << 6 | first block << 3 | second block);
+    // and whether some query's minimum was met in other blocks too
     float bound[4], best[4];
     int bblk[4];
-    bool tie[4];
+    bool tie = false;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         bound[j] = __shfl_sync(0xffffffffu, act ? own : -1.0f, (lane & ~3) + j);
         best[j] = INFINITY;
         bblk[j] = -1;
-        tie[j] = false;
     }
     // the box of the quad's queries and their largest bound, and the tile's
     float3 slo = make_float3(INFINITY, INFINITY, INFINITY);
@@ -975,15 +982,30 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     const float3 qlo = make_float3(warp_min(slo.x), warp_min(slo.y), warp_min(slo.z));
     const float3 qhi = make_float3(warp_max(shi.x), warp_max(shi.y), warp_max(shi.z));
     const float R = fmaxf(warp_max(sR), 0.0f);
-    auto eval = [&](const float4* blk, int b) {
+    // one block of 8, or two at once (their minimum is folded once)
+    auto eval = [&](const float4* blk, int code) {
         const float2* P = reinterpret_cast<const float2*>(blk) + t;
         const float2 px = P[0], py = P[4], pz = P[8];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float2 d = dist2x2(px, py, pz, nx[j], ny[j], nz[j]);
             const float m = fminf(d.x, d.y);
-            tie[j] = tie[j] || m == best[j];
-            bblk[j] = m < best[j] ? b : bblk[j];
+            tie |= m == best[j];
+            bblk[j] = m < best[j] ? code : bblk[j];
+            best[j] = fminf(best[j], m);
+        }
+    };
+    auto eval2 = [&](const float4* ba, const float4* bb, int code) {
+        const float2* P = reinterpret_cast<const float2*>(ba) + t;
+        const float2* Q = reinterpret_cast<const float2*>(bb) + t;
+        const float2 px = P[0], py = P[4], pz = P[8], qx = Q[0], qy = Q[4], qz = Q[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 d = dist2x2(px, py, pz, nx[j], ny[j], nz[j]);
+            const float2 f = dist2x2(qx, qy, qz, nx[j], ny[j], nz[j]);
+            const float m = min3(fminf(d.x, d.y), f.x, f.y);
+            tie |= m == best[j];
+            bblk[j] = m < best[j] ? code : bblk[j];
             best[j] = fminf(best[j], m);
         }
     };
@@ -995,18 +1017,16 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     {
         const int grp = lane >> 3, sub = lane & 7;
         for (int s = 0; s < C.nb2 && !wide; s += 32) {
-            const int i2 = s + lane;
-            bool hit = false;
-            if (i2 < C.nb2)
-                hit = box_bound(qlo, qhi, __ldg(C.box2 + 2 * i2), __ldg(C.box2 + 2 * i2 + 1)) <= R;
-            unsigned m2 = __ballot_sync(0xffffffffu, hit);
+            const int i2 = s + lane, c2 = min(i2, C.nb2 - 1);
+            const float l2 = box_bound(qlo, qhi, __ldg(C.box2 + 2 * c2), __ldg(C.box2 + 2 * c2 + 1));
+            unsigned m2 = __ballot_sync(0xffffffffu, (l2 <= R) & (i2 < C.nb2));
             wide = __popc(m2) > WIDE_BOX2;
             while (m2 && !wide) {
                 const int t2 = take4(m2, grp);
-                const int i1 = (s + t2) * 8 + sub;
-                hit = false;
-                if (t2 >= 0 && i1 < C.nb1)
-                    hit = box_bound(qlo, qhi, __ldg(C.box1 + 2 * i1), __ldg(C.box1 + 2 * i1 + 1)) <= R;
+                const int i1 = (s + t2) * 8 + sub, c1 = min(max(i1, 0), C.nb1 - 1);
+                const float l1 =
+                    box_bound(qlo, qhi, __ldg(C.box1 + 2 * c1), __ldg(C.box1 + 2 * c1 + 1));
+                const bool hit = (l1 <= R) & (t2 >= 0) & (i1 < C.nb1);
                 const unsigned m1 = __ballot_sync(0xffffffffu, hit);
                 if (hit) sw.hit[hits + __popc(m1 & ((1u << lane) - 1u))] = i1;
                 hits += __popc(m1);
@@ -1019,7 +1039,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     if (!wide) {
         auto stage = [&](int h) {
             if (h < hits) {
-                TreeStage& st = sw.stage[h % STAGES];
+                TreeStage& st = sw.stage[h & (STAGES - 1)];
                 const int b1 = sw.hit[h];
                 const float4* P = C.pts + 64LL * b1;
                 copy16(&st.pts[lane], P + lane);
@@ -1034,23 +1054,25 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
             copy_wait<STAGES - 2>();
             __syncwarp();  // the stage has landed for every lane, and the one before is done with
             stage(h + STAGES - 1);
-            const TreeStage& st = sw.stage[h % STAGES];
-            const int first = 8 * sw.hit[h];
+            const TreeStage& st = sw.stage[h & (STAGES - 1)];
+            const int b1 = sw.hit[h];
             // each box of 8 against the queries of each quad: lane t tests boxes t and t + 4
-            const bool hit0 =
-                first + t < C.nb && box_bound(slo, shi, st.box[2 * t], st.box[2 * t + 1]) <= sR;
-            const bool hit1 = first + t + 4 < C.nb &&
-                              box_bound(slo, shi, st.box[2 * t + 8], st.box[2 * t + 9]) <= sR;
-            unsigned m0 = __ballot_sync(0xffffffffu, hit0), m1 = __ballot_sync(0xffffffffu, hit1);
-            if (!(m0 | m1)) continue;
-            m0 |= m0 >> 16, m1 |= m1 >> 16;  // bits t of all quads together
-            m0 |= m0 >> 8, m1 |= m1 >> 8;
-            m0 = ((m0 | (m0 >> 4)) & 0xfu) | (((m1 | (m1 >> 4)) & 0xfu) << 4);
+            const float l0 = box_bound(slo, shi, st.box[2 * t], st.box[2 * t + 1]);
+            const float l1 = box_bound(slo, shi, st.box[2 * t + 8], st.box[2 * t + 9]);
+            unsigned m = __reduce_or_sync(
+                0xffffffffu, (l0 <= sR ? 1u << t : 0u) | (l1 <= sR ? 16u << t : 0u));
+            if (!m) continue;
             do {
-                const int c = __ffs(m0) - 1;
-                eval(st.pts + 8 * c, first + c);
-                m0 &= m0 - 1;
-            } while (m0);
+                const int c = __ffs(m) - 1;
+                m &= m - 1;
+                if (m) {
+                    const int d = __ffs(m) - 1;
+                    m &= m - 1;
+                    eval2(st.pts + 8 * c, st.pts + 8 * d, (b1 << 6) | (c << 3) | d);
+                } else {
+                    eval(st.pts + 8 * c, (b1 << 6) | (c << 3) | c);
+                }
+            } while (m);
             const bool better = best[0] < bound[0] || best[1] < bound[1] || best[2] < bound[2] ||
                                 best[3] < bound[3];
             if (__any_sync(0xffffffffu, better)) {
@@ -1070,21 +1092,24 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     // place in the sorted order; lane t keeps those of the quad's t-th query, its own.
     float md = own;
     int nn = 0x7fffffff, at = 0;
-    bool alone = valid && (wide || !act);
+    const unsigned tied = __ballot_sync(0xffffffffu, tie) >> (lane & ~3);
+    const bool alone = valid && (wide || !act || (tied & 0xfu) != 0);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         float v = best[j];
         v = fminf(v, __shfl_xor_sync(0xffffffffu, v, 1));
         v = fminf(v, __shfl_xor_sync(0xffffffffu, v, 2));
-        int i = 0x7fffffff, p = 8 * bblk[j] + 2 * t;
+        int i = 0x7fffffff, p = 0;
         if (bblk[j] >= 0 && best[j] == v) {
-            const float2* P = reinterpret_cast<const float2*>(C.pts + 8LL * bblk[j]) + t;
-            const float2 d = dist2x2(__ldg(P), __ldg(P + 4), __ldg(P + 8), nx[j], ny[j], nz[j]);
-            const float2 id = __ldg(P + 12);
-            if (d.x == v) i = __float_as_int(id.x);
-            if (d.y == v && __float_as_int(id.y) < i) {
-                i = __float_as_int(id.y);
-                ++p;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int b = 8 * (bblk[j] >> 6) + ((h ? bblk[j] : bblk[j] >> 3) & 7);
+                const float2* P = reinterpret_cast<const float2*>(C.pts + 8LL * b) + t;
+                const float2 d = dist2x2(__ldg(P), __ldg(P + 4), __ldg(P + 8), nx[j], ny[j], nz[j]);
+                const float2 id = __ldg(P + 12);
+                const int ix = __float_as_int(id.x), iy = __float_as_int(id.y);
+                if (d.x == v && ix < i) i = ix, p = 8 * b + 2 * t;
+                if (d.y == v && iy < i) i = iy, p = 8 * b + 2 * t + 1;
             }
         }
         const int mine = i;
@@ -1093,9 +1118,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
         // indices are distinct: one lane holds the minimum
         const unsigned holds = __ballot_sync(0xffffffffu, mine == i) >> (lane & ~3);
         p = __shfl_sync(0xffffffffu, p, (lane & ~3) + ((__ffs(holds) - 1) & 3));
-        const unsigned tm = __ballot_sync(0xffffffffu, tie[j] && best[j] == v);
         if (t == j) {
-            alone = alone || (valid && ((tm >> (lane & ~3)) & 0xfu) != 0);
             nn = i;
             at = p;
             md = fminf(md, v);
