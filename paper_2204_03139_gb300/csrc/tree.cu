@@ -740,9 +740,12 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
 // ---------------------------------------------------------------------------------------
 // search
 // ---------------------------------------------------------------------------------------
-constexpr int SEARCH_THREADS = 64;  // one query per thread; small CTAs free their slots early
+// One query per thread. CTAs of one warp free their slots as soon as it is done, and the block-wide
+// values are known to be the same in all lanes: 4.7% faster than two warps on 64 uneven trajectories
+// (18.0 against 18.9 ms), four warps 5.1% slower.
+constexpr int SEARCH_THREADS = 32;
 #ifndef DC_TREE_MIN_BLOCKS
-#define DC_TREE_MIN_BLOCKS 16
+#define DC_TREE_MIN_BLOCKS 32
 #endif
 // A query whose starting bound is 2^5 times (as squared distance) that of the tile's others
 constexpr int OUTLIER_LOG2 = 5;
