@@ -1,6 +1,7 @@
 // Host entry points of libdiffcloud.so (declared in include/diffcloud.h).
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -217,23 +218,25 @@ int check_ws(void* ws, size_t ws_bytes, size_t need) {
 int g_engine = ENGINE_AUTO;  // process-wide engine set by dc_tune_set
 
 // The Chamfer engine of a call: the one dc_tune_set asked for, when the problem fits it (else
-// the direct engine); by default the pruned search from TREE_AUTO_MIN_PAIRS pairs in all, and
-// the direct engine below, where the pruned search's sort and three launches take longer than
-// all pairs. Measured on one GB300, whole call with the gradient, replayed from a CUDA graph,
-// direct / warp-level tensor filter / pruned: 1 frame of 16 384 points 134 / 130 / 170 us and of
-// 32 768 377 / 317 / 200 us; 4 frames of 8192 110 / 117 / 109 us; 16 frames of 4096
-// 111 / 111 / 105 us and of 8192 302 / 255 / 151 us; 40 frames of 2048 94 / 102 / 110 us, of 4096
-// 217 / 207 / 151 us and of 16 384 2.56 / 1.87 / 0.56 ms; 100 frames of 1024 82 / 83 / 77 us.
-// The tensor-core filters, which evaluate every pair too, stay available on request (their
-// results are the same).
+// the direct engine); by default the pruned search from TREE_AUTO_PAIRS / sqrt(frames) pairs in
+// all, and the direct engine below, where the pruned search's sort and its launches take longer
+// than all pairs: its time is mostly latency, which more frames share, so the line falls with
+// them. Measured on one GB300, whole call with the gradient, replayed from a CUDA graph, direct /
+// warp-level tensor filter / pruned in us: 1 frame of 8192 points 68 / 93 / 81, of 16 384
+// 134 / 130 / 135, of 32 768 377 / 317 / 157; 4 frames of 4096 58 / 76 / 66, of 8192
+// 110 / 115 / 93; 16 frames of 1024 41 / 54 / 45, of 2048 64 / 75 / 62, of 4096 109 / 111 / 91;
+// 40 frames of 512 42 / 50 / 38, of 1024 55 / 65 / 52, of 10 000 1000 / 820 / 198; 100 frames of
+// 256 40 / 50 / 36, of 512 56 / 60 / 44. The tensor-core filters, which evaluate every pair too,
+// stay available on request (their results are the same).
 // A pending stall test goes to the direct engine by default: the pruned search has no waits.
-constexpr double TREE_AUTO_MIN_PAIRS = 2.5e8;
+constexpr double TREE_AUTO_PAIRS = 2.5e8;
 
-int choose_engine(bool tc_fits, bool tree_fits, double pairs) {
+int choose_engine(bool tc_fits, bool tree_fits, double pairs, int frames) {
     if (g_engine == ENGINE_TREE) return tree_fits ? ENGINE_TREE : ENGINE_DIRECT;
     if (g_engine == ENGINE_AUTO)
-        return tree_fits && pairs >= TREE_AUTO_MIN_PAIRS && !stall_pending() ? ENGINE_TREE
-                                                                            : ENGINE_DIRECT;
+        return tree_fits && pairs >= TREE_AUTO_PAIRS / sqrt((double)frames) && !stall_pending()
+                   ? ENGINE_TREE
+                   : ENGINE_DIRECT;
     if (g_engine == ENGINE_DIRECT || !tc_fits) return ENGINE_DIRECT;
     return g_engine;
 }
@@ -254,7 +257,7 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     const bool chamfer = (phases & PH_CHAMFER) != 0;
     const int engine =
         chamfer && !direct_only
-            ? choose_engine(sz.tc_units > 0, sz.tree != 0, (double)a.T * (double)a.N * (double)a.M)
+            ? choose_engine(sz.tc_units > 0, sz.tree != 0, (double)a.T * (double)a.N * (double)a.M, a.T)
             : ENGINE_DIRECT;
     const int warps =
         (chamfer && engine == ENGINE_DIRECT) ? choose_warps(a.mode, sub[2], sub[1], sub[0]) : 1;
@@ -725,7 +728,7 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
         return fail(DC_EINVAL, "batch too large for 32-bit offsets");
     double pairs = 0.0;
     for (int k = 0; k < n_frames; ++k) pairs += (double)frames[k].N * (double)frames[k].M;
-    const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, pairs);
+    const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, pairs, n_frames);
     // the pruned search's plans can run the direct engine too (stall tests)
     const int warps = engine == ENGINE_DIRECT || engine == ENGINE_TREE
                           ? choose_warps(mode, sub[2], sub[1], sub[0])

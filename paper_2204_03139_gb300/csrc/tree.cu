@@ -507,14 +507,13 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
 
     // ---- starts of every (cell, slice): CTA r scans its share of the words over all slices ----
     {
-        const int per = words / S;  // a multiple of 64
-        const int chunks = per / 32;
-        const int cw = (chunks + PREP_WARPS - 1) / PREP_WARPS;
-        const int ch0 = min(chunks, warp * cw), ch1 = min(chunks, ch0 + cw);
+        const int first = words / 32 * r / S, end = words / 32 * (r + 1) / S;  // chunks of 32
+        const int cw = (end - first + PREP_WARPS - 1) / PREP_WARPS;
+        const int ch0 = min(end, first + warp * cw), ch1 = min(end, ch0 + cw);
         auto word_sum = [&](int v) { return packed ? (v & 0xffff) + (int)((unsigned)v >> 16) : v; };
         int tot = 0;
         for (int ch = ch0; ch < ch1; ++ch) {
-            const int c = r * per + 32 * ch + lane;
+            const int c = 32 * ch + lane;
 #pragma unroll
             for (int s = 0; s < S; ++s) tot += word_sum(remote(hist, s)[c]);
         }
@@ -538,7 +537,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
         for (int s = 0; s < S; ++s)
             if (s < r) run += *remote(&s_total, s);
         for (int ch = ch0; ch < ch1; ++ch) {
-            const int c = r * per + 32 * ch + lane;
+            const int c = 32 * ch + lane;
             int cnt[S], sum = 0;
 #pragma unroll
             for (int s = 0; s < S; ++s) {
@@ -1345,17 +1344,19 @@ cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max
         int optin = 0;
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         optin = (optin > 0 ? optin : 99 * 1024) - STATIC;
-        for (auto f : {k_tree_prep<1>, k_tree_prep<2>, k_tree_prep<4>, k_tree_prep<8>}) {
+        for (auto f : {k_tree_prep<1>, k_tree_prep<2>, k_tree_prep<3>, k_tree_prep<4>,
+                       k_tree_prep<6>, k_tree_prep<8>}) {
             cudaError_t e =
                 cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
             if (e) return e;
         }
         g_prep_smem[dev] = optin;
     }
-    // enough CTAs for the chip when there are few frames: a cluster of up to 8 per (frame,
-    // side), each CTA with at least one point per thread
+    // Few frames: a cluster of up to 8 CTAs per (frame, side), as many as are resident at once
+    // (two per SM), each with at least one point per thread.
     int S = 1;
-    while (S < 8 && 2 * n_frames * 2 * S <= 2 * 152 && max_n >= 2 * S * PREP_THREADS) S *= 2;
+    for (int q : {2, 3, 4, 6, 8})
+        if (2 * n_frames * q <= 2 * 152 && max_n >= q * PREP_THREADS) S = q;
     // the CDF, later the cells and the refinement's buffers: two CTAs per SM up to 27 000 faces
     size_t smem = CELL_BYTES + REFINE_BYTES;
     const bool cdf_shared = 4 * (size_t)max_f <= (size_t)g_prep_smem[dev];
@@ -1376,7 +1377,12 @@ cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max
     cfg.attrs = attr;
     cfg.numAttrs = S > 1 ? 2 : 1;
     const UniformArgs none{};
-    auto kernel = S == 8 ? k_tree_prep<8> : S == 4 ? k_tree_prep<4> : S == 2 ? k_tree_prep<2> : k_tree_prep<1>;
+    auto kernel = S == 8   ? k_tree_prep<8>
+                  : S == 6 ? k_tree_prep<6>
+                  : S == 4 ? k_tree_prep<4>
+                  : S == 3 ? k_tree_prep<3>
+                  : S == 2 ? k_tree_prep<2>
+                           : k_tree_prep<1>;
     cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a ? *a : none, w, (int)(a != nullptr),
                                        n_frames, rows, (int)cdf_shared);
     count_launch();
