@@ -227,7 +227,8 @@ int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream);
  *     bounding boxes of runs of 8, 64 and 512 points; a query evaluates the direct form only for
  *     boxes that its minimum so far does not exclude. Clouds of at most 2 097 152 points.
  *     DC_ENGINE_AUTO takes it for calls (and batch plans) of T frames with at least
- *     2.5e8 / sqrt(T) pairs in all, else the direct engine.
+ *     2.5e8 / sqrt(T) pairs in all (1.2e8 / sqrt(T) in dc_chamfer_fwd) and 300 pairs per point,
+ *     else the direct engine.
  *   DC_ENGINE_TENSOR -- a tensor-core filter: the expanded form |p|^2 - 2 p.q + |q|^2 on
  *     split-fp16 operands, warp-level MMAs (16 points x 8 candidates each), keeps per point
  *     and quarter of the candidates the three best blocks of 128, and the direct form

@@ -2,8 +2,7 @@
 
 The shapes it chooses between:
   ("pruned", 0)  the pruned search over sorted points and bounding boxes (clouds of at most
-                 2 097 152 points; the library's default for calls of T frames with 2.5e8 / sqrt(T)
-                 pairs and more);
+                 2 097 152 points; the library's default for larger calls, see diffcloud.h);
   ("tensor", 0)  the tensor-core filter on warp-level MMAs (frames of at most 524 288
                  points per side);
   ("tcgen05", 0) the same filter on tcgen05 MMAs;

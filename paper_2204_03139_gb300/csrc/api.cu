@@ -218,25 +218,37 @@ int check_ws(void* ws, size_t ws_bytes, size_t need) {
 int g_engine = ENGINE_AUTO;  // process-wide engine set by dc_tune_set
 
 // The Chamfer engine of a call: the one dc_tune_set asked for, when the problem fits it (else
-// the direct engine); by default the pruned search from TREE_AUTO_PAIRS / sqrt(frames) pairs in
-// all, and the direct engine below, where the pruned search's sort and its launches take longer
-// than all pairs: its time is mostly latency, which more frames share, so the line falls with
-// them. Measured on one GB300, whole call with the gradient, replayed from a CUDA graph, direct /
-// warp-level tensor filter / pruned in us: 1 frame of 8192 points 68 / 93 / 81, of 16 384
-// 134 / 130 / 135, of 32 768 377 / 317 / 157; 4 frames of 4096 58 / 76 / 66, of 8192
-// 110 / 115 / 93; 16 frames of 1024 41 / 54 / 45, of 2048 64 / 75 / 62, of 4096 109 / 111 / 91;
-// 40 frames of 512 42 / 50 / 38, of 1024 55 / 65 / 52, of 10 000 1000 / 820 / 198; 100 frames of
-// 256 40 / 50 / 36, of 512 56 / 60 / 44. The tensor-core filters, which evaluate every pair too,
-// stay available on request (their results are the same).
+// the direct engine). By default the pruned search when
+//   - it has TREE_AUTO_PAIRS / sqrt(frames) pairs in all (TREE_AUTO_PAIRS_POINTS when the sim
+//     points are given): its sort and launches are mostly latency, which more frames share, so
+//     the line falls with them; and
+//   - TREE_AUTO_PAIRS_PER_QUERY pairs per query: a query costs about as much as that many pairs
+//     of the direct engine (100 frames of 20 000 points against 300: 299 us, direct 271);
+// and the direct engine below. Measured on one GB300, replayed from a CUDA graph, direct /
+// warp-level tensor filter / pruned in us, sampled with the gradient: 1 frame of 8192 points
+// 68 / 93 / 81, of 16 384 134 / 130 / 135, of 32 768 377 / 317 / 157; 4 frames of 4096
+// 58 / 76 / 66, of 8192 110 / 115 / 93; 16 frames of 1024 41 / 54 / 45, of 2048 64 / 75 / 62, of
+// 4096 109 / 111 / 91; 40 frames of 1024 55 / 65 / 52, of 10 000 1000 / 820 / 198; 100 frames of
+// 1024 81 / 81 / 62. Given points (uniform in a cube), direct / pruned: 1 frame of 16 384
+// 104 / 62; 4 of 8192 97 / 64; 7 of 4097 x 3001 60 / 51; 16 of 2048 53 / 49; 40 of 1024 44 / 48,
+// of 2048 83 / 59. The tensor-core filters, which evaluate every pair too, stay available on
+// request (their results are the same).
 // A pending stall test goes to the direct engine by default: the pruned search has no waits.
 constexpr double TREE_AUTO_PAIRS = 2.5e8;
+constexpr double TREE_AUTO_PAIRS_POINTS = 1.2e8;
+constexpr double TREE_AUTO_PAIRS_PER_QUERY = 300.0;
 
-int choose_engine(bool tc_fits, bool tree_fits, double pairs, int frames) {
+int choose_engine(bool tc_fits, bool tree_fits, double pairs, double queries, int frames,
+                  bool points) {
     if (g_engine == ENGINE_TREE) return tree_fits ? ENGINE_TREE : ENGINE_DIRECT;
-    if (g_engine == ENGINE_AUTO)
-        return tree_fits && pairs >= TREE_AUTO_PAIRS / sqrt((double)frames) && !stall_pending()
+    if (g_engine == ENGINE_AUTO) {
+        const double least = (points ? TREE_AUTO_PAIRS_POINTS : TREE_AUTO_PAIRS) /
+                             sqrt((double)frames);
+        return tree_fits && pairs >= least && pairs >= TREE_AUTO_PAIRS_PER_QUERY * queries &&
+                       !stall_pending()
                    ? ENGINE_TREE
                    : ENGINE_DIRECT;
+    }
     if (g_engine == ENGINE_DIRECT || !tc_fits) return ENGINE_DIRECT;
     return g_engine;
 }
@@ -257,7 +269,8 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     const bool chamfer = (phases & PH_CHAMFER) != 0;
     const int engine =
         chamfer && !direct_only
-            ? choose_engine(sz.tc_units > 0, sz.tree != 0, (double)a.T * (double)a.N * (double)a.M, a.T)
+            ? choose_engine(sz.tc_units > 0, sz.tree != 0, (double)a.T * (double)a.N * (double)a.M,
+                            (double)a.T * ((double)a.N + (double)a.M), a.T, a.pts != nullptr)
             : ENGINE_DIRECT;
     const int warps =
         (chamfer && engine == ENGINE_DIRECT) ? choose_warps(a.mode, sub[2], sub[1], sub[0]) : 1;
@@ -726,9 +739,12 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
     long long sub[3];
     if (!batch_sizes(frames, n_frames, sz, sub))
         return fail(DC_EINVAL, "batch too large for 32-bit offsets");
-    double pairs = 0.0;
-    for (int k = 0; k < n_frames; ++k) pairs += (double)frames[k].N * (double)frames[k].M;
-    const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, pairs, n_frames);
+    double pairs = 0.0, queries = 0.0;
+    for (int k = 0; k < n_frames; ++k) {
+        pairs += (double)frames[k].N * (double)frames[k].M;
+        queries += (double)frames[k].N + (double)frames[k].M;
+    }
+    const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, pairs, queries, n_frames, false);
     // the pruned search's plans can run the direct engine too (stall tests)
     const int warps = engine == ENGINE_DIRECT || engine == ENGINE_TREE
                           ? choose_warps(mode, sub[2], sub[1], sub[0])

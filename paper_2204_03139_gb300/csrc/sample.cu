@@ -256,13 +256,13 @@ __device__ void area_cdf(const AreaFrame& fr, int* err) {
     const int f0 = min(F, tid * per), f1 = min(F, f0 + per);
     bool bad_idx = false, bad_val = false;
 
+    // the area weights in face order (neighbouring threads read neighbouring faces; a thread's
+    // own segment of faces was a stride of per x 12 bytes between the lanes of a warp)
+    for (int f = tid; f < F; f += CDF_THREADS)
+        cdf[f] = face_weight(verts, faces, mask, V, f, bad_idx, bad_val);
+    __syncthreads();
     FF v = {0.0f, 0.0f};
-    // pass 1: the segment's area weights, kept in the thread's own slots of the CDF buffer
-    for (int f = f0; f < f1; ++f) {
-        const float a = face_weight(verts, faces, mask, V, f, bad_idx, bad_val);
-        cdf[f] = a;
-        v = ff_add1(v, a);
-    }
+    for (int f = f0; f < f1; ++f) v = ff_add1(v, cdf[f]);
 
     // block-wide inclusive scan of the segment sums
 #pragma unroll
@@ -287,7 +287,7 @@ __device__ void area_cdf(const AreaFrame& fr, int* err) {
     FF run = warp > 0 ? ff_add(s_w[warp - 1], ex) : ex;
 
     for (int f = f0; f < f1; ++f) {
-        run = ff_add1(run, cdf[f]);  // pass 2 reads back this thread's own area weights
+        run = ff_add1(run, cdf[f]);
         cdf[f] = run.hi;
     }
     if (bad_idx || bad_val) set_status(err, DC_EINVAL);
