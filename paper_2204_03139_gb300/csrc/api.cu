@@ -65,7 +65,7 @@ Layout make_layout(const Sizes& s) {
     L.nnba = take(s.cols * 4);
     L.loss = take(s.n_frames * 4);
     L.part = take(s.n_frames * s.slices * 2 * 4);
-    L.frame_err = take(s.n_frames * 8);
+    L.frame_err = take(s.n_frames * (s.tree ? 8 : 4));
     L.fbox = take(s.n_frames * 16);
     const long long tcp = s.tc_units > 0 ? s.rows + s.cols : 0;  // points with forms
     L.tc_ufr = take(s.tc_units * 4);
@@ -816,7 +816,6 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
         d.cdf0 = cdf0;
         d.v0 = v0;
         d.unit0 = unit;
-        d.tc_unit0 = tunit;
         fd[k] = d;
         if (keyed(engine)) {
             // sim rows against the targets, then (Eq. 1) the targets against the sim points

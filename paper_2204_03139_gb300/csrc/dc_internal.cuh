@@ -167,7 +167,6 @@ struct FrameDesc {
     int v0;               // offset of this frame's vertices in the gradient accumulators
     int unit0;            // first Chamfer unit of this frame
     int skip;             // weight (or gradient multiplier) 0: no work, L reported as 0
-    int tc_unit0;         // first tensor-core unit of this frame (sim rows, then targets)
 };
 
 // Header at the start of every workspace.

@@ -26,7 +26,7 @@ __device__ __forceinline__ void frame_scales(const UniformArgs& a, int k, float&
     }
 }
 
-// The record of frame k of a uniform trajectory (unit0 and tc_unit0 left at 0).
+// The record of frame k of a uniform trajectory (unit0 left at 0).
 __device__ __forceinline__ FrameDesc uniform_frame(const UniformArgs& a, const Ws& w, int k) {
     const int Npad = round_up(a.N, ROW_PAD), Mpad = round_up(a.M, COL_PAD);
     FrameDesc f;
@@ -60,7 +60,6 @@ __device__ __forceinline__ FrameDesc uniform_frame(const UniformArgs& a, const W
     f.cdf0 = k * a.F;
     f.v0 = k * a.V;
     f.unit0 = 0;
-    f.tc_unit0 = 0;
     return f;
 }
 

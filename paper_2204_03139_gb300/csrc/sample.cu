@@ -226,10 +226,7 @@ __device__ void build_uniform(const UniformArgs& a, const Ws& w) {
     }
     // unit0 now holds "live frames before"; restore its documented meaning
     __syncthreads();
-    for (int k = tid; k < a.T; k += nt) {
-        w.frames[k].unit0 = k * upf;
-        w.frames[k].tc_unit0 = k * tupf;
-    }
+    for (int k = tid; k < a.T; k += nt) w.frames[k].unit0 = k * upf;
 }
 
 __global__ void __launch_bounds__(BUILD_THREADS) k_build_uniform(UniformArgs a, Ws w) {
