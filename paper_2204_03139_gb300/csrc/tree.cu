@@ -1263,20 +1263,34 @@ constexpr int OUT_THREADS = 256;
 // per coordinate and (point, target) pair the points' sums save half the scatter, and vectors
 // two thirds of the rest (64 uneven trajectories: 3.8 ms as one epilogue, 1.5 ms here).
 __global__ void __launch_bounds__(OUT_THREADS) k_tree_out(Ws w, int n_frames, int slices, int lanes,
-                                                          int loss_blocks, int bidir) {
+                                                          int loss_blocks, int steps, int bidir) {
     pdl_entry();
     const int tid = threadIdx.x;
     if ((int)blockIdx.x >= loss_blocks) {
-        const int step = blockIdx.x - loss_blocks;
-        const FrameDesc* fr = w.frames + w.step_frame[step];
-        if (fr->skip || !fr->grad || !fr->verts) return;
-        const int g = step * TREE_STEP + tid, p = g - fr->row0;
-        if (p >= fr->N) return;
-        const float4 gr = w.tgx[g];
-        const int i = __float_as_int(__ldg(w.tpts + 4LL * fr->row0 + 32LL * (p >> 3) + 24 + (p & 7)));
-        const int4 q = __ldg(w.fw + fr->row0 + i);
-        if (q.x < 0) return;
-        scatter_face(w, fr, q, gr);
+        // two steps per block, so that two chains of dependent loads overlap
+        const FrameDesc* fr[2];
+        float4 g[2];
+        int4 q[2];
+        int i[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int step = 2 * (blockIdx.x - loss_blocks) + h;
+            fr[h] = w.frames + w.step_frame[min(step, steps - 1)];
+            const int at = step * TREE_STEP + tid, p = at - fr[h]->row0;
+            q[h].x = -1;
+            i[h] = -1;
+            if (step < steps && !fr[h]->skip && fr[h]->grad && fr[h]->verts && p < fr[h]->N) {
+                g[h] = w.tgx[at];
+                i[h] = __float_as_int(
+                    __ldg(w.tpts + 4LL * fr[h]->row0 + 32LL * (p >> 3) + 24 + (p & 7)));
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (i[h] >= 0) q[h] = __ldg(w.fw + fr[h]->row0 + i[h]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (q[h].x >= 0) scatter_face(w, fr[h], q[h], g[h]);
         return;
     }
     __shared__ float s_red[2][OUT_THREADS / 8];
@@ -1407,8 +1421,10 @@ cudaError_t launch_tree_out(const Ws& w, int n_frames, int slices, int lanes, in
                             int mode, float* total, cudaStream_t s) {
     const int bidir = mode == DC_BIDIR_MEAN;
     const int loss_blocks = div_up(n_frames * slices, OUT_THREADS / lanes);
-    cudaError_t e = launch_pdl(k_tree_out, loss_blocks + (max_v > 0 ? rows / TREE_STEP : 0),
-                               OUT_THREADS, 0, s, w, n_frames, slices, lanes, loss_blocks, bidir);
+    const int steps = rows / TREE_STEP;
+    cudaError_t e = launch_pdl(k_tree_out, loss_blocks + (max_v > 0 ? div_up(steps, 2) : 0),
+                               OUT_THREADS, 0, s, w, n_frames, slices, lanes, loss_blocks, steps,
+                               bidir);
     count_launch();
     if (!e && max_v > 0) e = launch_grad_out(w, n_frames, max_v, s);
     return e ? e : launch_frame_loss(w, n_frames, slices, bidir, total, s);

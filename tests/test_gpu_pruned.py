@@ -117,3 +117,49 @@ def test_device_errors_reach_the_status():
         with autotune.tuned(PRUNED), pytest.raises(_lib.DCError) as e:
             _lib.dc_loss_traj(v.to(DEV), f.to(DEV), d.to(DEV), y.to(DEV), check=True)
         assert e.value.code == code
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("T,n,m", [(1, 1, 1), (1, 513, 255), (3, 1025, 257), (5, 2000, 3001)])
+def test_recomputing_backward_equals_the_forward_gradient(T, n, m, mode):
+    """dc_loss_traj_bwd with the neighbours of a forward call gives that call's gradient. Both sum
+    the same float32 contributions in another order and grouping: a few roundings (6e-8) each."""
+    tr = W.lift_trajectory(3, 13, T, n, m, name="b")
+    v, f = torch.from_numpy(tr.verts).to(DEV), torch.from_numpy(tr.faces).to(DEV)
+    d, y = (torch.from_numpy(np.ascontiguousarray(x)).to(DEV)
+            for x in (tr.draws_tn3(), tr.targets_tm3()))
+    w = torch.linspace(0.0, 1.5, T, device=DEV) if T > 1 else None  # the first frame is skipped
+    for shape in (PRUNED, DIRECT):
+        with autotune.tuned(shape):
+            r = _lib.dc_loss_traj(v, f, d, y, mode=mode, frame_w=w, check=True)
+        g = _lib.dc_loss_traj_bwd(v, f, d, y, r["nn_ab"], r["nn_ba"], mode=mode, frame_w=w,
+                                  grad_total=torch.ones(1, device=DEV), check=True)
+        assert parity.rel_l2(g.cpu(), r["grad_verts"].cpu()) < 2e-6
+    # a neighbour out of range is reported
+    bad = r["nn_ab"].clone()
+    bad[-1, -1] = m
+    with pytest.raises(_lib.DCError) as e:
+        _lib.dc_loss_traj_bwd(v, f, d, y, bad, r["nn_ba"], mode=mode, frame_w=w,
+                              grad_total=torch.ones(1, device=DEV), check=True)
+    assert e.value.code == _lib.DC_EINVAL
+
+
+@pytest.mark.timeout(120)
+def test_stall_test_runs_the_direct_engine_where_the_pruned_search_is_the_default():
+    """The pruned search has no bounded waits to run out, so a pending stall test sends the call
+    (or the run of a plan) that would take it to the direct engine, whose waits give up."""
+    from paper_2204_03139_gb300.batch import BatchedLoss, DeviceTrajectory
+
+    tr = W.lift_trajectory(6, 20, 40, 2000, 2100, name="s")
+    v, f = torch.from_numpy(tr.verts).to(DEV), torch.from_numpy(tr.faces).to(DEV)
+    d, y = (torch.from_numpy(np.ascontiguousarray(x)).to(DEV)
+            for x in (tr.draws_tn3(), tr.targets_tm3()))
+    plan = BatchedLoss([DeviceTrajectory.from_host(tr, DEV)], shape=PRUNED)
+    for run in (lambda: _lib.dc_loss_traj(v, f, d, y, check=True)["loss_frames"],
+                lambda: (plan.run(check=True), plan.loss_frames[0])[1]):
+        good = run().clone()
+        _lib.test_inject_stall()
+        with pytest.raises(_lib.DCError) as e:
+            run()
+        assert e.value.code == _lib.DC_ETIMEOUT
+        assert torch.equal(run(), good)
