@@ -214,7 +214,7 @@ int dc_batch_plan_async(const dc_frame* frames, int n_frames, int mode, void* ws
 
 /*
  * dc_batch_run -- forward (and the gradient of every frame whose grad_verts is set) of a
- * planned batch: sampling, one persistent Chamfer launch over all frames, neighbours,
+ * planned batch: sampling, the nearest-neighbour launches over all frames, neighbours,
  * losses, gradient scatter. loss_total [1] out, nullable: sum of w L over the frames.
  * Reads only device memory, so the launch sequence can be captured in a CUDA graph.
  */
@@ -225,10 +225,13 @@ int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream);
  * (the float32 direct form, lowest index among equal distances):
  *   DC_ENGINE_PRUNED -- the points of both clouds sorted along a space-filling curve, with
  *     bounding boxes of runs of 8, 64 and 512 points; a query evaluates the direct form only for
- *     boxes that its minimum so far does not exclude. Clouds of at most 2 097 152 points.
- *     DC_ENGINE_AUTO takes it for calls (and batch plans) of T frames with at least
- *     2.5e8 / sqrt(T) pairs in all (1.2e8 / sqrt(T) in dc_chamfer_fwd) and 300 pairs per point,
- *     else the direct engine.
+ *     boxes that its minimum so far does not exclude. Clouds of at most 2 097 152 points, and
+ *     at most about 1.5 faces per point where DC_ENGINE_AUTO would not take it.
+ *     DC_ENGINE_AUTO takes it for calls (and batch plans) of at least 7e7 pairs (Eq. 2: 9.5e7)
+ *     plus 9600 per point of the largest side, 250 per point, 600 + F / 8 per face of the largest
+ *     mesh of F faces and 10 per face in all (up to 5 times as many in Eq. 2 with over 3 targets per sim point);
+ *     else the warp-level tensor filter from 1e9 pairs and 5e7 per frame on, and the direct
+ *     engine below.
  *   DC_ENGINE_TENSOR -- a tensor-core filter: the expanded form |p|^2 - 2 p.q + |q|^2 on
  *     split-fp16 operands, warp-level MMAs (16 points x 8 candidates each), keeps per point
  *     and quarter of the candidates the three best blocks of 128, and the direct form
@@ -254,7 +257,7 @@ enum {
 
 typedef struct dc_tune {
     int32_t warps_per_cta; /* direct engine: 0 (automatic), 1, 2 or 4 */
-    int32_t engine;        /* DC_ENGINE_AUTO, _DIRECT, _TENSOR or _TCGEN05 */
+    int32_t engine;        /* DC_ENGINE_AUTO, _DIRECT, _TENSOR, _TCGEN05 or _PRUNED */
 } dc_tune;
 
 int dc_tune_set(const dc_tune* tune); /* NULL restores automatic */
@@ -316,9 +319,11 @@ int dc_fp32_fma_rate(int packed, int iters, double* flop_per_s, dc_stream_t stre
 
 /*
  * dc_test_inject_stall -- for testing the failure detection (the paper has no counterpart).
- * The next Chamfer launch in the process never requests the first target chunk of each CTA,
- * so the bounded waits on it give up after 2 s: the call completes, its workspace reports
- * DC_ETIMEOUT (dc_ws_status), and the device stays usable for the next call.
+ * The next nearest-neighbour launch of an engine with bounded waits (all but the pruned search)
+ * in the process never requests the first target chunk of each CTA, so the waits on it give up
+ * after 2 s: the call completes, its workspace reports DC_ETIMEOUT (dc_ws_status), and the
+ * device stays usable for the next call. While it is pending, calls under DC_ENGINE_AUTO and
+ * runs of planned batches take the direct engine instead of the pruned search.
  */
 int dc_test_inject_stall(void);
 

@@ -57,8 +57,6 @@ Layout make_layout(const Sizes& s) {
     L.cdf = take(s.sum_f * 4);
     L.x = take(s.rows * 16);
     L.fw = take(s.rows * 16);
-    L.tsoa = take(6 * s.cols * 4);
-    L.tpl = take(3 * s.cols * 4);
     L.pab = take(s.rows * 8);
     L.pba = take(s.cols * 8);
     L.nnab = take(s.rows * 4);
@@ -67,6 +65,8 @@ Layout make_layout(const Sizes& s) {
     L.part = take(s.n_frames * s.slices * 2 * 4);
     L.frame_err = take(s.n_frames * (s.tree ? 8 : 4));
     L.fbox = take(s.n_frames * 16);
+    L.tsoa = take(6 * s.cols * 4);
+    L.tpl = take(3 * s.cols * 4);
     const long long tcp = s.tc_units > 0 ? s.rows + s.cols : 0;  // points with forms
     L.tc_ufr = take(s.tc_units * 4);
     L.tc_urb = take(s.tc_units * 4);
@@ -78,11 +78,15 @@ Layout make_layout(const Sizes& s) {
     L.kpart = take(s.tc_units > 0 ? s.tc_slots * 2 * TC_UNIT_ROWS * TC_KEYS * 4 : 0);
     L.tcfb = take(tcp * 4);
     L.tcfn = take(s.tc_units > 0 ? s.n_frames * 8 : 0);
+    const size_t other_end = off;
+    // A call runs one engine, so the pruned search's regions share the memory of the others'
+    // target planes and tensor-core regions.
+    off = L.tsoa;
     const long long tp = s.tree ? s.rows + s.cols : 0;
+    L.y = take(s.tree ? s.cols * 16 : 0);
     L.step_frame = take(tp / TREE_STEP * 4);
     L.tkey = take(tp * 4);
     L.tord = take(tp * 8);
-    L.y = take(s.tree ? s.cols * 16 : 0);
     L.tpts = take(tp * 16);
     L.tkb = take(tp / 8 * 4);
     L.tbox = take(tp / 8 * 32);
@@ -91,7 +95,7 @@ Layout make_layout(const Sizes& s) {
     L.frec = take(s.tree ? s.sum_f * 48 : 0);
     L.tgx = take(s.tree ? s.rows * 16 : 0);
     L.grad4 = take(s.tree ? s.sum_v * 16 : 0);
-    L.total = off;
+    L.total = std::max(off, other_end);
     return L;
 }
 
@@ -164,6 +168,66 @@ bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
 constexpr long long INT_LIMIT = 0x7fffffffLL;
 
+// What the default rule of the engines looks at.
+struct Load {
+    double pairs = 0, rows = 0, cols = 0;  // sums over the frames
+    double side = 0, sides = 0;            // largest side of a frame; sum of the larger sides
+    double faces = 0, face_sum = 0;        // largest mesh; sum over the frames
+
+    void add(double n, double m, double f, double frames) {
+        pairs += frames * n * m;
+        rows += frames * n;
+        cols += frames * m;
+        side = std::max(side, std::max(n, m));
+        sides += frames * std::max(n, m);
+        faces = std::max(faces, f);
+        face_sum += frames * f;
+    }
+};
+
+// The default rule: the pruned search takes problems of at least this many pairs. Against the
+// direct engine it has fixed costs (its launches, worth 7e7 pairs; in Eq. 2, whose direct pass is
+// cheaper, 9.5e7), the latency of sorting the largest side (9600 pairs per point), and work per
+// point (250) and per face (600 for each of the largest mesh, more where its areas fill the shared
+// memory of the preparation's CTAs, and 10 for each in all). Where Eq. 2 has few
+// queries against many targets, the 32 queries of a tile lie far apart and share little, so it
+// takes up to 5 times as many pairs from 3 targets per query on. The line was laid through 11 384
+// random problems of 1 to 100 frames of 300 to 33 000 points a side (sampled and given points,
+// both modes, one GB300, direct and pruned replayed from a CUDA graph), those nearest to it: of
+// the 4292 it gives to the pruned search 8 take over 3% longer there (7% at most) than before
+// (direct, or the tensor-core filter by its rule below), and on average they take 0.62 of it; a
+// line that only counted pairs would have 1651 of 8823 take longer, up to 5.2 times. Of the ones
+// it leaves, 30% would gain 10% or more, but lie among others that lose. Direct / pruned in us:
+// 1 frame of 16 384 points 134 / 135, of 32 768 377 / 157; 16 frames of 2048 64 / 62, of 4096
+// 109 / 91; 40 of 10 000 1000 / 198; 10 of 9400 against 1200 81 / 93; 6 of 741 against 28 000 (Eq. 2)
+// 64 / 261. Many faces: 16 frames of 4096 points, 8 per point 261 / 345; 40 of 8192, 8 per point
+// 1049 / 526.
+double tree_pairs(const Load& l, int mode) {
+    const bool uni = mode == DC_UNIDIR_SUM;
+    const double thin = uni && l.cols > 3 * l.rows
+                            ? std::min(5.0, 1 + (l.cols / l.rows - 3) / 4)
+                            : 1.0;
+    return thin * ((uni ? 9.5e7 : 7e7) + 9600 * l.side + 250 * l.sides +
+                   (600 + l.faces / 8) * l.faces + 10 * l.face_sum);
+}
+
+// The pruned search's regions are kept when they need no more memory than the other engines do
+// (up to about 1.5 faces per point), or when the problem is one that the default rule gives to
+// it: elsewhere (say 60 000 faces for 40 points) the face records would multiply the workspace.
+bool keep_tree(Sizes s, const Load& l) {
+    if (l.pairs >= tree_pairs(l, DC_BIDIR_MEAN)) return true;  // the lower of the modes' lines
+    const size_t with = make_layout(s).total;
+    s.tree = 0;
+    return with <= make_layout(s).total;
+}
+
+// a mesh of one face stands for given points (dc_chamfer_fwd)
+Load uniform_load(int T, int F, int N, int M) {
+    Load l;
+    l.add(N, M, F > 1 ? F : 0, T);
+    return l;
+}
+
 // Sizes of a uniform trajectory; false if any derived count overflows int32. The unit
 // arrays are sized for the narrowest CTA (the most units); sub[w] is the Chamfer work
 // (sub-chunks) at CTA width 1, 2 and 4 (indices 0, 1, 2).
@@ -195,6 +259,7 @@ bool uniform_sizes(int T, int V, int F, int N, int M, Sizes& s, long long sub[3]
         if (chunks >= INT_LIMIT) return false;
         s.tc_slots = tc_grid(chunks);  // the pass's CTAs (partial-key slots are per CTA)
     }
+    if (s.tree) s.tree = keep_tree(s, uniform_load(T, F, N, M));
     return s.rows < INT_LIMIT && s.cols < INT_LIMIT && s.sum_f < INT_LIMIT &&
            sub[0] < INT_LIMIT && s.rows * 3 < INT_LIMIT * 16 && s.cols * 6 < INT_LIMIT * 16 &&
            3LL * V < INT_LIMIT && (s.rows + s.cols) * 2 < INT_LIMIT;
@@ -218,35 +283,21 @@ int check_ws(void* ws, size_t ws_bytes, size_t need) {
 int g_engine = ENGINE_AUTO;  // process-wide engine set by dc_tune_set
 
 // The Chamfer engine of a call: the one dc_tune_set asked for, when the problem fits it (else
-// the direct engine). By default the pruned search when
-//   - it has TREE_AUTO_PAIRS / sqrt(frames) pairs in all (TREE_AUTO_PAIRS_POINTS when the sim
-//     points are given): its sort and launches are mostly latency, which more frames share, so
-//     the line falls with them; and
-//   - TREE_AUTO_PAIRS_PER_QUERY pairs per query: a query costs about as much as that many pairs
-//     of the direct engine (100 frames of 20 000 points against 300: 299 us, direct 271);
-// and the direct engine below. Measured on one GB300, replayed from a CUDA graph, direct /
-// warp-level tensor filter / pruned in us, sampled with the gradient: 1 frame of 8192 points
-// 68 / 93 / 81, of 16 384 134 / 130 / 135, of 32 768 377 / 317 / 157; 4 frames of 4096
-// 58 / 76 / 66, of 8192 110 / 115 / 93; 16 frames of 1024 41 / 54 / 45, of 2048 64 / 75 / 62, of
-// 4096 109 / 111 / 91; 40 frames of 1024 55 / 65 / 52, of 10 000 1000 / 820 / 198; 100 frames of
-// 1024 81 / 81 / 62. Given points (uniform in a cube), direct / pruned: 1 frame of 16 384
-// 104 / 62; 4 of 8192 97 / 64; 7 of 4097 x 3001 60 / 51; 16 of 2048 53 / 49; 40 of 1024 44 / 48,
-// of 2048 83 / 59. The tensor-core filters, which evaluate every pair too, stay available on
-// request (their results are the same).
-// A pending stall test goes to the direct engine by default: the pruned search has no waits.
-constexpr double TREE_AUTO_PAIRS = 2.5e8;
-constexpr double TREE_AUTO_PAIRS_POINTS = 1.2e8;
-constexpr double TREE_AUTO_PAIRS_PER_QUERY = 300.0;
+// the direct engine). By default the pruned search by the rule above; what it leaves goes to the
+// warp-level tensor filter from TC_AUTO_PAIRS pairs in all and TC_AUTO_PAIRS_PER_FRAME per frame on
+// (few queries' worth of pairs or very many faces: the filter's fixed launches are paid back
+// there, 4 frames of 32 768 points 0.856 against 1.051 ms direct, one frame of 16 384 139
+// against 119 us), and to the direct engine below. A pending stall test goes to these: the pruned
+// search has no waits.
+constexpr double TC_AUTO_PAIRS = 1e9;
+constexpr double TC_AUTO_PAIRS_PER_FRAME = 5e7;
 
-int choose_engine(bool tc_fits, bool tree_fits, double pairs, double queries, int frames,
-                  bool points) {
+int choose_engine(bool tc_fits, bool tree_fits, const Load& l, int frames, int mode) {
     if (g_engine == ENGINE_TREE) return tree_fits ? ENGINE_TREE : ENGINE_DIRECT;
     if (g_engine == ENGINE_AUTO) {
-        const double least = (points ? TREE_AUTO_PAIRS_POINTS : TREE_AUTO_PAIRS) /
-                             sqrt((double)frames);
-        return tree_fits && pairs >= least && pairs >= TREE_AUTO_PAIRS_PER_QUERY * queries &&
-                       !stall_pending()
-                   ? ENGINE_TREE
+        if (tree_fits && l.pairs >= tree_pairs(l, mode) && !stall_pending()) return ENGINE_TREE;
+        return tc_fits && l.pairs >= TC_AUTO_PAIRS && l.pairs >= TC_AUTO_PAIRS_PER_FRAME * frames
+                   ? ENGINE_TC
                    : ENGINE_DIRECT;
     }
     if (g_engine == ENGINE_DIRECT || !tc_fits) return ENGINE_DIRECT;
@@ -269,8 +320,8 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     const bool chamfer = (phases & PH_CHAMFER) != 0;
     const int engine =
         chamfer && !direct_only
-            ? choose_engine(sz.tc_units > 0, sz.tree != 0, (double)a.T * (double)a.N * (double)a.M,
-                            (double)a.T * ((double)a.N + (double)a.M), a.T, a.pts != nullptr)
+            ? choose_engine(sz.tc_units > 0, sz.tree != 0, uniform_load(a.T, a.F, a.N, a.M), a.T,
+                            a.mode)
             : ENGINE_DIRECT;
     const int warps =
         (chamfer && engine == ENGINE_DIRECT) ? choose_warps(a.mode, sub[2], sub[1], sub[0]) : 1;
@@ -652,6 +703,7 @@ int dc_loss_traj_bwd(const float* verts, const int32_t* faces, const uint8_t* fa
 static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
     s = Sizes{n, 0, 0, 0, 0, epilogue_slices(n), 0, 0, 1, 0};
     sub[0] = sub[1] = sub[2] = 0;
+    Load load;
     long long max_v = 0, tc_units = 0, tc_chunks = 0;
     bool tc_fits = true;
     for (int k = 0; k < n; ++k) {
@@ -667,6 +719,7 @@ static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
         if (fr[k].grad_verts && fr[k].V > max_v) max_v = fr[k].V;
         tc_fits = tc_fits && Npad <= TC_MAX_COLS && Mpad <= TC_MAX_COLS;
         if (fr[k].N > TREE_MAX_POINTS || fr[k].M > TREE_MAX_POINTS) s.tree = 0;
+        load.add(fr[k].N, fr[k].M, fr[k].F, 1);
         const long long u0 = div_up(fr[k].N, TC_UNIT_ROWS), u1 = div_up(fr[k].M, TC_UNIT_ROWS);
         tc_units += u0 + u1;
         tc_chunks += u0 * (Mpad / TC_CHUNK) + u1 * (Npad / TC_CHUNK);
@@ -676,6 +729,7 @@ static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
         s.tc_units = tc_units;
         s.tc_slots = tc_grid(tc_chunks);
     }
+    if (s.tree) s.tree = keep_tree(s, load);
     return s.rows < INT_LIMIT && s.cols < INT_LIMIT && s.sum_f < INT_LIMIT &&
            sub[0] < INT_LIMIT && s.n_units < INT_LIMIT && s.cols * 6 < INT_LIMIT * 16 &&
            3 * max_v < INT_LIMIT && tc_chunks < INT_LIMIT && (s.rows + s.cols) * 2 < INT_LIMIT;
@@ -739,12 +793,9 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
     long long sub[3];
     if (!batch_sizes(frames, n_frames, sz, sub))
         return fail(DC_EINVAL, "batch too large for 32-bit offsets");
-    double pairs = 0.0, queries = 0.0;
-    for (int k = 0; k < n_frames; ++k) {
-        pairs += (double)frames[k].N * (double)frames[k].M;
-        queries += (double)frames[k].N + (double)frames[k].M;
-    }
-    const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, pairs, queries, n_frames, false);
+    Load load;
+    for (int k = 0; k < n_frames; ++k) load.add(frames[k].N, frames[k].M, frames[k].F, 1);
+    const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, load, n_frames, mode);
     // the pruned search's plans can run the direct engine too (stall tests)
     const int warps = engine == ENGINE_DIRECT || engine == ENGINE_TREE
                           ? choose_warps(mode, sub[2], sub[1], sub[0])

@@ -163,3 +163,22 @@ def test_stall_test_runs_the_direct_engine_where_the_pruned_search_is_the_defaul
             run()
         assert e.value.code == _lib.DC_ETIMEOUT
         assert torch.equal(run(), good)
+
+
+@pytest.mark.parametrize("grid,engine", [(45, _lib.ENGINE_PRUNED), (182, _lib.ENGINE_DIRECT)])
+def test_many_faces_per_point_leave_the_default_to_the_direct_engine(grid, engine):
+    """16 frames of 4096 x 4096 points: with 1/2 face per point the pruned search is the default,
+    with 8 its face records cost more than they save. The losses are the same either way."""
+    tr = W.lift_trajectory(9, grid, 16, 4096, 4096, name="f")
+    v, f = torch.from_numpy(tr.verts).to(DEV), torch.from_numpy(tr.faces).to(DEV)
+    d, y = (torch.from_numpy(np.ascontiguousarray(x)).to(DEV)
+            for x in (tr.draws_tn3(), tr.targets_tm3()))
+    ws = _lib.workspace(_lib.dc_workspace_size(16, v.shape[1], f.shape[0], 4096, 4096), DEV)
+    r = _lib.dc_loss_traj(v, f, d, y, out={"ws": ws}, check=True)
+    assert int(ws[52:56].cpu().view(torch.int32)[0]) == engine  # the header's engine word
+    for shape in (PRUNED, DIRECT):
+        with autotune.tuned(shape):
+            ref = _lib.dc_loss_traj(v, f, d, y, check=True)
+        for k in ("loss_frames", "loss_total", "nn_ab", "nn_ba"):
+            assert torch.equal(r[k], ref[k])
+        assert parity.rel_l2(r["grad_verts"].cpu(), ref["grad_verts"].cpu()) < 1e-6
