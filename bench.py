@@ -2,8 +2,8 @@
 
 One step (the default workload, batched_uneven) = the loss and every vertex gradient of 64
 cloth trajectories of uneven sizes (grids 15x15 to 80x80, 20 to 100 frames, 2 000 to 30 000
-target points per frame): area CDFs, sampling, one persistent nearest-neighbour launch over
-all frames, neighbour recovery, losses and the adjoint scatter, planned once at the
+target points per frame): area CDFs, sampling, the nearest-neighbour search over all
+frames, losses and the adjoint scatter, planned once at the
 autotuned shape and replayed from a CUDA graph. The metric is point pairs per second (one
 pair = one (sim point, target point) distance of Eq. 1). `--workload trajectory_50x50`
 times one dc_loss_traj call over the 40-frame 50x50 trajectory instead.
@@ -43,8 +43,12 @@ MMA_SYNC_TFLOPS = 600.0
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none \
 #       -k 'regex:k_tcpass$' -s 3 -c 1 python bench.py --workload trajectory_50x50 --steps 3 \
 #       --warmup 3 --no-cpu-baseline [--mode eq2]  (and --workload trajectory_100x100;
-#       -k regex:k_chamfer for --workload single_frame)
-CHAMFER_TRAFFIC_BYTES = {("batched_uneven", "k_tcpass", "eq1"): 7.72e9 + 5.41e9,
+#       -k regex:k_chamfer for --workload single_frame, -k regex:k_tree_search and --shape
+#       pruned:0 for the pruned search)
+CHAMFER_TRAFFIC_BYTES = {("batched_uneven", "k_tree_search", "eq1"): 6.27e9 + 2.46e9,
+                         ("trajectory_50x50", "k_tree_search", "eq1"): 26.60e6,
+                         ("trajectory_50x50", "k_tree_search", "eq2"): 22.91e6,
+                         ("batched_uneven", "k_tcpass", "eq1"): 7.72e9 + 5.41e9,
                          ("trajectory_50x50", "k_tcpass", "eq1"): 53.58e6 + 8.11e6,
                          ("trajectory_50x50", "k_tcpass", "eq2"): 26.11e6 + 0.04e6,
                          ("trajectory_100x100", "k_tcpass", "eq1"): 431.75e6 + 281.22e6,
@@ -55,7 +59,7 @@ CHAMFER_TRAFFIC_BYTES = {("batched_uneven", "k_tcpass", "eq1"): 7.72e9 + 5.41e9,
                          ("trajectory_50x50", "k_chamfer<false>", "eq2"): 19.57e6}
 
 
-def pruned_roof(points, queries, kernel_s, launch_pairs):
+def pruned_roof(points, queries, kernel_s, launch_pairs, traffic=None):
     """Roofline entry of the pruned search (k_tree_search and k_tree_single). It evaluates the
     direct form only for boxes of 8 points that the query's minimum so far does not exclude
     (about 180 pairs per query on these clouds), so the 8-flop accounting of all pairs does not
@@ -65,7 +69,7 @@ def pruned_roof(points, queries, kernel_s, launch_pairs):
     hbm = measured_peaks().get("hbm_gbs")
     gbs = nbytes / kernel_s / 1e9 if kernel_s else None
     return {"bound": "issue", "achieved": gbs, "peak": hbm, "unit": "GB/s",
-            "frac": gbs / hbm if (gbs and hbm) else None, "traffic": None,
+            "frac": gbs / hbm if (gbs and hbm) else None, "traffic": traffic,
             "kernel": "k_tree_search + k_tree_single",
             "kernel_ms": kernel_s * 1e3 if kernel_s else None,
             "pairs_per_s_kernel": launch_pairs / kernel_s if kernel_s else None,
@@ -519,7 +523,9 @@ def run_gpu(args, rank, world, dist):
             "pairs_per_s_kernel": pairs / chamfer_avg_s if chamfer_n else None}
     if engine == _lib.ENGINE_PRUNED:
         roof = pruned_roof(T * (N + M), T * (N + (M if mode == _lib.BIDIR_MEAN else 0)),
-                           chamfer_avg_s, pairs)
+                           chamfer_avg_s, pairs,
+                           CHAMFER_TRAFFIC_BYTES.get((args.workload, "k_tree_search", args.mode))
+                           if args.frames is None else None)
         achieved = None
     best_fma = max(fma.values()) / 1e12
     roof["peak_measured"] = {
@@ -762,7 +768,9 @@ def run_batched(args, rank, world, dist):
     if shape[0] == "pruned":
         pts = sum(int(t.n_off[-1]) + int(t.m_off[-1]) for t in trajs)
         q = pts if mode == _lib.BIDIR_MEAN else sum(int(t.n_off[-1]) for t in trajs)
-        roof = pruned_roof(pts, q, ck, pairs)
+        roof = pruned_roof(pts, q, ck, pairs,
+                           CHAMFER_TRAFFIC_BYTES.get(("batched_uneven", "k_tree_search", args.mode))
+                           if args.batch_trajectories is None else None)
     if tc:
         # the pass evaluates each pair once per direction on the tensor cores: one m16n8k16
         # MMA (4096 flop) per 128 pairs, in both directions for Eq. 1

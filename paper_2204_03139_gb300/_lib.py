@@ -421,9 +421,8 @@ def dc_loss_traj_noalloc(verts, faces, draws, targets, mode=BIDIR_MEAN, frame_w=
 
 def tune_set(warps_per_cta: int = 0, engine: int = ENGINE_AUTO):
     """Nearest-neighbour engine (ENGINE_AUTO, ENGINE_DIRECT, ENGINE_TENSOR, ENGINE_TCGEN05 or
-    ENGINE_PRUNED)
-    and the direct engine's CTA width (1, 2 or 4 warps; 0: automatic) for every later call
-    and plan."""
+    ENGINE_PRUNED) and the direct engine's CTA width (1, 2 or 4 warps; 0: automatic) for every
+    later call and plan."""
     t = dc_tune(int(warps_per_cta), int(engine))
     _check(lib().dc_tune_set(ctypes.byref(t)))
 

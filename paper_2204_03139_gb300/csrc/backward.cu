@@ -7,7 +7,8 @@
 // targets chose it, and both sums use 16-byte vector atomics: a target costs one of them and a sim
 // point three, instead of nine scalar atomics each. Bound by the L2's random accesses (the
 // neighbour gathers and the atomics). 100 frames of 32 768 points against as many targets: the
-// general staging and epilogue, which this replaces, took 138 + 404 us.
+// general staging and epilogue, which this replaces, took 138 + 404 us; the rows here 145, the
+// columns 42, the scatter 63 and the copy out 9 us.
 #include <algorithm>
 
 #include "dc_sampling.cuh"

@@ -1,4 +1,6 @@
-// Tensor-core filter of the brute-force nearest-neighbour search (Eq. 1, Eq. 2).
+// Tensor-core filter of the brute-force nearest-neighbour search (Eq. 1, Eq. 2). By default
+// large calls take the pruned search (tree.cu) and small ones the direct form; these engines run on
+// request and for the large calls that the pruned search's rule leaves.
 //
 // Every row point (the sim points, and in Eq. 1 also the targets) is compared with every
 // column point of its frame (the targets, respectively the sim points) through the

@@ -304,8 +304,16 @@ __device__ __forceinline__ int cell_get(const int* h, bool packed, int c) {
 //   2. curve keys; histogram of their top bits (cells) in shared memory
 //   3. scan over cells and slices (through distributed shared memory), scatter of the points'
 //      keys and indices
-//   4. each point's rank within its cell by its whole key; the sorted points as blocks of 8 (x[8] y[8] z[8] index[8], one 128-byte line)
+//   4. each point's rank within its cell by its whole key; the sorted points as blocks of 8
+//      (x[8] y[8] z[8] index[8], one 128-byte line)
 //   5. bounding boxes of 8, 64 and 512 consecutive points
+// Bound by latency: chains of dependent gathers (face pick, corners) and one block-wide meeting
+// per phase. 40 frames of 10 000 points against as many: 61 us at 36% of the load pipe, its warps
+// waiting 5.3 cycles per instruction for memory and 3.6 at barriers. One kernel for all phases
+// keeps the counters and the draws' points on chip; clusters of 3 instead of 2 for those 80 sides
+// (240 CTAs instead of 160) 210 -> 198 us per call. 64 uneven trajectories, 1.14e8 points:
+// 6.1 ms with 1024 threads and gathers from global memory, 5.0 ms with face records and two
+// points per step, 4.5 ms with the ring below.
 template <int S>
 __global__ void __launch_bounds__(PREP_THREADS, 2)
     k_tree_prep(UniformArgs a, Ws w, int uniform, int n_frames, int rows, int cdf_shared) {
@@ -883,6 +891,12 @@ __device__ __forceinline__ TreeCols tree_cols(const Ws& w, const FrameDesc* fr, 
 //   - Queries that would widen the walk of the others (outliers: a bound far above theirs), all
 //     queries of a tile that meets too many boxes, and queries that met their minimum in two
 //     blocks (exact ties, whose lowest index must win) are queued for k_tree_single.
+// Bound by instruction issue and the load pipe: 2650 instructions per tile, of which about 20
+// blocks of 8 evaluated (50 each) and 9 boxes of 64 staged are most; 69% of issue slots, 55% of
+// the load pipe's wavefronts, 2.5 cycles per instruction waiting for memory. 40 frames of 10 000
+// points against as many: 94 us, where evaluating every pair takes 630 us (tensor-core filter)
+// or 943 us (direct form). 64 uneven trajectories: 10.8 ms (one query per lane 11.5 ms and
+// 3.8 ms in k_tree_single, without the gradient's sums), the tensor-core filter 158 ms.
 __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     k_tree_search(Ws w, int rows, int bidir) {
     pdl_wait();
@@ -1156,7 +1170,10 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
 }
 
 // The queued queries, one warp each: the same walk with the query's own box (a point), every
-// lane one point of four blocks of 8.
+// lane one point of four blocks of 8. Bound by latency (three levels of dependent loads, 12.6
+// cycles per instruction), so 64 warps per SM at 32 registers, although that spills: with 42 or
+// 51 registers (48 and 40 warps) the 100-frame call of 32 768 points takes 1770 and 1784 us
+// instead of 1755. 64 uneven trajectories 0.96 ms, 40 frames of 10 000 points 30 us.
 constexpr int SINGLE_THREADS = 128;
 __global__ void __launch_bounds__(SINGLE_THREADS, 16) k_tree_single(Ws w, int rows, int bidir) {
     pdl_wait();
@@ -1261,7 +1278,8 @@ constexpr int OUT_THREADS = 256;
 // face's vertices with the barycentric weights (Eq. 4), 16 bytes per vertex. In sorted order
 // neighbouring points share faces and vertices, so the face look-ups hit L1; against one atomic
 // per coordinate and (point, target) pair the points' sums save half the scatter, and vectors
-// two thirds of the rest (64 uneven trajectories: 3.8 ms as one epilogue, 1.5 ms here).
+// two thirds of the rest (64 uneven trajectories: 3.8 ms as one epilogue, 1.4 ms here). Bound by
+// the latency of its gathers and the L2's atomics (40 frames of 10 000 points: 21 us, of 20 MB).
 __global__ void __launch_bounds__(OUT_THREADS) k_tree_out(Ws w, int n_frames, int slices, int lanes,
                                                           int loss_blocks, int steps, int bidir) {
     pdl_entry();

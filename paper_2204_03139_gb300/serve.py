@@ -9,10 +9,10 @@ every optimisation). The server batches continuously:
     the device once, on a copy stream, and stay resident until the result is delivered;
   - time slicing: an admitted request is cut into items of consecutive frames of at most
     `item_pairs` point pairs, so that a long request cannot hold the GPU for its whole
-    duration (one persistent Chamfer launch occupies every SM until it ends);
+    duration (a batch's nearest-neighbour launch occupies every SM until it ends);
   - batching: whenever one of the compute streams is free, admitted items of the same mode, up
     to `max_batch_pairs`, go into one planned launch sequence (dc_batch_plan / dc_batch_run):
-    one persistent Chamfer launch covers all their frames, whatever their sizes. Requests are
+    its launches cover all their frames, whatever their sizes. Requests are
     served shortest remaining work first (a short request passes a long one; long ones run
     one after another instead of sharing the GPU and all finishing late), except that a
     request waiting longer than `max_wait_s` goes first, so that long ones never starve;
