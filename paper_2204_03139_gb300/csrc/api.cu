@@ -195,7 +195,8 @@ struct Load {
 // random problems of 1 to 100 frames of 300 to 33 000 points a side (sampled and given points,
 // both modes, one GB300, direct and pruned replayed from a CUDA graph), those nearest to it: of
 // the 4292 it gives to the pruned search 8 take over 3% longer there (7% at most) than before
-// (direct, or the tensor-core filter by its rule below), and on average they take 0.62 of it; a
+// (direct, or the tensor-core filter by its rule below), and on average they take 0.62 of it (7085
+// more, drawn afterwards: 8, 9% at most, 0.60); a
 // line that only counted pairs would have 1651 of 8823 take longer, up to 5.2 times. Of the ones
 // it leaves, 30% would gain 10% or more, but lie among others that lose. Direct / pruned in us:
 // 1 frame of 16 384 points 134 / 135, of 32 768 377 / 157; 16 frames of 2048 64 / 62, of 4096
@@ -310,6 +311,14 @@ int keyed_grid(int engine, long long chunks) {
 
 constexpr int MAX_GRID_Y = 65535;
 
+// The recomputing backward of its own (backward.cu) from this many points per frame or in all on: it
+// is two launches more than the staging kernel and epilogue. Graph replays in us, the general
+// kernels / backward.cu: 5 frames of 1000 points a side 16.7 / 20.9, 1 of 2048 16.6 / 18.6, 20 of 2000
+// and 500 23.0 / 27.0; 40 of 1000 27.1 / 27.1, 75 of 1000 27.7 / 28.5, 1 of 8000 28.6 / 24.5, 100 of
+// 2000 55.6 / 45.5.
+constexpr long long BWD_FRAME_POINTS = 16000;
+constexpr long long BWD_POINTS = 200000;
+
 int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total, void* ws,
                 size_t ws_bytes, cudaStream_t st, bool direct_only = false) {
     Sizes sz;
@@ -339,7 +348,9 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     // with sampling to follow, the tables and the area CDFs (and the frame boxes of the
     // tensor-core forms) share one launch
     const bool fused = (phases & PH_AREA) && (phases & PH_SAMPLE);
-    if (a.bwd && sz.tree && a.T <= MAX_GRID_Y) {
+    const long long points = (long long)a.N + a.M;
+    if (a.bwd && sz.tree && a.T <= MAX_GRID_Y &&
+        (points >= BWD_FRAME_POINTS || a.T * points >= BWD_POINTS)) {
         cudaError_t e = launch_backward(a, w, st);
         return e ? cuda_fail(e, "kernel launch") : DC_OK;
     }

@@ -120,7 +120,8 @@ def test_device_errors_reach_the_status():
 
 
 @pytest.mark.parametrize("mode", [0, 1])
-@pytest.mark.parametrize("T,n,m", [(1, 1, 1), (1, 513, 255), (3, 1025, 257), (5, 2000, 3001)])
+@pytest.mark.parametrize("T,n,m", [(1, 1, 1), (1, 513, 255), (3, 1025, 257), (5, 2000, 3001),
+                                   (2, 15745, 255), (2, 257, 15744), (103, 1025, 975)])
 def test_recomputing_backward_equals_the_forward_gradient(T, n, m, mode):
     """dc_loss_traj_bwd with the neighbours of a forward call gives that call's gradient. Both sum
     the same float32 contributions in another order and grouping: a few roundings (6e-8) each."""
