@@ -80,7 +80,8 @@ class BatchedLoss:
         shape (autotune.SHAPES); otherwise the library's default. outputs: per trajectory a
         (loss_frames [T], grad_verts [T, V, 3] or None) pair of device tensors to write into
         instead of new ones. async_plan: upload the plan from pinned staging memory without
-        waiting for the stream (the staging stays referenced by this object)."""
+        waiting for the stream (the staging outlives the upload, also if this object does
+        not)."""
         from . import autotune
 
         self.trajs = list(trajs)
@@ -173,6 +174,11 @@ class BatchedLoss:
                                               ctypes.c_void_p(self.ws.data_ptr()), nb,
                                               ctypes.c_void_p(self._staging.data_ptr()), sb,
                                               ctypes.c_void_p(self.stream.cuda_stream)))
+            # The library queued the upload, so torch's pinned allocator does not know that the
+            # stream still reads the staging; a copy of torch's own from it (into the total,
+            # which a run overwrites) tells it. The block then goes to nobody else before the
+            # upload has completed, also when this object is dropped right after run().
+            self.total.view(torch.uint8).copy_(self._staging[:4], non_blocking=True)
         else:
             _lib._check(L.dc_batch_plan(self.frames, nfr, mode,
                                         ctypes.c_void_p(self.ws.data_ptr()), nb,
