@@ -63,7 +63,10 @@ enum {
 };
 
 /* Bytes of workspace the uniform-trajectory entry points need for T frames of V vertices,
- * F faces, N samples and M target points (M may be 0 for dc_sample). */
+ * F faces, N samples and M target points (M may be 0 for dc_sample). With more than about 1.5
+ * faces per point this counts the regions of the pruned search only where DC_ENGINE_AUTO takes
+ * it, so a problem with fewer faces can be given more bytes; a workspace without room for these
+ * regions (one sized for a larger mesh, say) is accepted too, and the call runs another engine. */
 size_t dc_workspace_size(int T, int V, int F, int N, int M);
 
 /*
@@ -184,7 +187,8 @@ typedef struct dc_frame {
     int32_t* nn_ba;       /* [M] out, nullable */
 } dc_frame;
 
-/* Bytes of workspace a batch of n_frames frames needs. */
+/* Bytes of workspace a batch of n_frames frames needs (as for dc_workspace_size, a plan also
+ * accepts one without room for the pruned search's regions). */
 size_t dc_batch_workspace_size(const dc_frame* frames, int n_frames);
 
 /*

@@ -222,6 +222,16 @@ bool keep_tree(Sizes s, const Load& l) {
     return with <= make_layout(s).total;
 }
 
+// The layout of a call or plan in a workspace of ws_bytes: without the pruned search's regions
+// (and so on another engine) where only these do not fit. A workspace sized for a larger mesh may
+// be without them, since keep_tree drops them for face-heavy problems.
+Layout fit_layout(Sizes& s, size_t ws_bytes) {
+    const Layout L = make_layout(s);
+    if (!s.tree || ws_bytes >= L.total) return L;
+    s.tree = 0;
+    return make_layout(s);
+}
+
 // a mesh of one face stands for given points (dc_chamfer_fwd)
 Load uniform_load(int T, int F, int N, int M) {
     Load l;
@@ -326,6 +336,7 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     int spu = 0;
     if (!uniform_sizes(a.T, a.V, a.F, a.N, a.M, sz, sub, spu, !direct_only))
         return fail(DC_EINVAL, "problem too large for 32-bit offsets");
+    const Layout L = fit_layout(sz, ws_bytes);
     const bool chamfer = (phases & PH_CHAMFER) != 0;
     const int engine =
         chamfer && !direct_only
@@ -339,7 +350,6 @@ int run_uniform(UniformArgs a, unsigned phases, int epi_flags, float* loss_total
     a.units_per_frame = div_up(a.N, ROWS_PER_WARP * warps);
     a.subs_per_unit = spu;
     a.slices = (int)sz.slices;
-    const Layout L = make_layout(sz);
     int rc = check_ws(ws, ws_bytes, L.total);
     if (rc) return rc;
     const Ws w = make_ws(ws, L);
@@ -806,16 +816,20 @@ int plan_impl(const dc_frame* frames, int n_frames, int mode, void* ws, size_t w
         return fail(DC_EINVAL, "batch too large for 32-bit offsets");
     Load load;
     for (int k = 0; k < n_frames; ++k) load.add(frames[k].N, frames[k].M, frames[k].F, 1);
+    // (a size query answers for every workspace that a plan accepts)
+    const bool any_keyed =
+        keyed(choose_engine(sz.tc_units > 0, sz.tree != 0, load, n_frames, mode)) ||
+        keyed(choose_engine(sz.tc_units > 0, false, load, n_frames, mode));
+    const Layout L = size_only ? make_layout(sz) : fit_layout(sz, ws_bytes);
     const int engine = choose_engine(sz.tc_units > 0, sz.tree != 0, load, n_frames, mode);
     // the pruned search's plans can run the direct engine too (stall tests)
     const int warps = engine == ENGINE_DIRECT || engine == ENGINE_TREE
                           ? choose_warps(mode, sub[2], sub[1], sub[0])
                           : 1;
-    const Layout L = make_layout(sz);
     // the staging image: the table regions [hdr, cdf), then the tensor-core unit tables
     const size_t img_bytes = L.cdf + (keyed(engine) ? L.tca - L.tc_ufr : 0);
     if (size_only) {
-        *size_only = img_bytes;
+        *size_only = L.cdf + (any_keyed ? L.tca - L.tc_ufr : 0);
         return DC_OK;
     }
     int rc = check_ws(ws, ws_bytes, L.total);
