@@ -191,6 +191,11 @@ typedef struct dc_frame {
  * accepts one without room for the pruned search's regions). */
 size_t dc_batch_workspace_size(const dc_frame* frames, int n_frames);
 
+/* The fewest bytes that dc_batch_plan accepts for these frames: without the pruned search's
+ * regions. For callers with a budget of device memory; with fewer than about 1.5 faces per point it
+ * equals dc_batch_workspace_size. 0 if the frames are invalid. */
+size_t dc_batch_workspace_least(const dc_frame* frames, int n_frames);
+
 /*
  * dc_batch_plan -- validate the frames (host array), lay them out in ws and copy the
  * descriptor tables into it (a host-to-device copy on `stream`). The plan stays valid

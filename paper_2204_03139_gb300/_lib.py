@@ -77,6 +77,7 @@ def lib() -> ctypes.CDLL:
                 "dc_loss_traj_bwd": (I, [P, P, P, P, P, I, I, I, I, I, I, P, P, P, P, P, P, P,
                                          S, P]),
                 "dc_batch_workspace_size": (S, [P, I]),
+                "dc_batch_workspace_least": (S, [P, I]),
                 "dc_batch_plan": (I, [P, I, I, P, S, P]),
                 "dc_batch_plan_bytes": (S, [P, I, I]),
                 "dc_batch_plan_async": (I, [P, I, I, P, S, P, S, P]),

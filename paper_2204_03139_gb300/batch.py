@@ -74,14 +74,15 @@ class BatchedLoss:
 
     def __init__(self, trajs, mode=_lib.BIDIR_MEAN, weights=None, grad=True, graph=False,
                  nn=False, stream=None, tune=False, shape=None, outputs=None,
-                 async_plan=False):
+                 async_plan=False, spare=None):
         """tune=True: plan with the shape the autotuner found fastest for this batch's size
         bucket (timing every shape first if the bucket has no entry); shape: plan with this
         shape (autotune.SHAPES); otherwise the library's default. outputs: per trajectory a
         (loss_frames [T], grad_verts [T, V, 3] or None) pair of device tensors to write into
         instead of new ones. async_plan: upload the plan from pinned staging memory without
         waiting for the stream (the staging outlives the upload, also if this object does
-        not)."""
+        not). spare: device bytes that the workspace may take beyond the least it needs (default:
+        any); extra_bytes says how many of them it took."""
         from . import autotune
 
         self.trajs = list(trajs)
@@ -99,11 +100,11 @@ class BatchedLoss:
         # outputs and workspace belong to the batch's stream (the caching allocator reuses
         # memory per stream); the plan keeps the shape it was made with
         with torch.cuda.stream(self.stream), autotune.tuned(shape):
-            self._build(mode, weights, grad, nn, outputs, async_plan)
+            self._build(mode, weights, grad, nn, outputs, async_plan, spare)
         if graph:
             self._capture()
 
-    def _build(self, mode, weights, grad, nn, outputs=None, async_plan=False):
+    def _build(self, mode, weights, grad, nn, outputs=None, async_plan=False, spare=None):
         dev = self.device
         nfr = sum(t.T for t in self.trajs)
         # the dc_frame table, filled column by column (one row per frame)
@@ -161,6 +162,12 @@ class BatchedLoss:
         nb = int(L.dc_batch_workspace_size(self.frames, nfr))
         if nb == 0:
             raise _lib.DCError(_lib.DC_EINVAL, "bad batch sizes")
+        self.extra_bytes = 0
+        if spare is not None:
+            least = int(L.dc_batch_workspace_least(self.frames, nfr))
+            if nb - least > spare:
+                nb = least
+            self.extra_bytes = nb - least
         self.ws = torch.empty(nb, dtype=torch.uint8, device=dev)
         self.total = torch.empty(1, dtype=torch.float32, device=dev)
         self.workspace_bytes = nb

@@ -756,7 +756,7 @@ static bool batch_sizes(const dc_frame* fr, int n, Sizes& s, long long sub[3]) {
            3 * max_v < INT_LIMIT && tc_chunks < INT_LIMIT && (s.rows + s.cols) * 2 < INT_LIMIT;
 }
 
-size_t dc_batch_workspace_size(const dc_frame* frames, int n_frames) {
+static size_t batch_workspace(const dc_frame* frames, int n_frames, bool tree) {
     if (!frames || n_frames <= 0) return 0;
     for (int k = 0; k < n_frames; ++k)
         if (frames[k].N <= 0 || frames[k].M <= 0 || frames[k].F <= 0 || frames[k].V <= 0)
@@ -764,7 +764,16 @@ size_t dc_batch_workspace_size(const dc_frame* frames, int n_frames) {
     Sizes sz;
     long long sub[3];
     if (!batch_sizes(frames, n_frames, sz, sub)) return 0;
+    if (!tree) sz.tree = 0;
     return make_layout(sz).total;
+}
+
+size_t dc_batch_workspace_size(const dc_frame* frames, int n_frames) {
+    return batch_workspace(frames, n_frames, true);
+}
+
+size_t dc_batch_workspace_least(const dc_frame* frames, int n_frames) {
+    return batch_workspace(frames, n_frames, false);
 }
 
 int dc_batch_plan(const dc_frame* frames, int n_frames, int mode, void* ws, size_t ws_bytes,

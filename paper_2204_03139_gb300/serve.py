@@ -141,7 +141,9 @@ def request_bytes(traj, grad: bool = True) -> int:
     inputs = (traj.verts.nbytes + traj.faces.nbytes + traj.draws.nbytes + traj.targets.nbytes
               + traj.F)  # and the face mask, if any
     outputs = 4 * traj.T + (traj.verts.nbytes if grad else 0)
-    ws = int(_lib.lib().dc_batch_workspace_size(_frames_of(traj), traj.T))
+    # the least workspace: a batch takes more (for the pruned search of face-heavy meshes) only
+    # while the budget has room
+    ws = int(_lib.lib().dc_batch_workspace_least(_frames_of(traj), traj.T))
     if ws == 0:
         raise _lib.DCError(_lib.DC_EINVAL, "request sizes are invalid")
     return inputs + outputs + ws + 64 * 1024
@@ -168,6 +170,7 @@ class Server:
         self._waiting: collections.deque = collections.deque()
         self._admitted: list = []
         self._used = 0
+        self._extra = 0  # bytes of the running batches' workspaces beyond their least
         self._next_id = 0
         self._next_batch = 0
         self._closing = False
@@ -250,7 +253,8 @@ class Server:
     def _admit(self):
         while True:
             with self._cv:
-                if not self._waiting or self._used + self._waiting[0].nbytes > self.budget:
+                if (not self._waiting or
+                        self._used + self._extra + self._waiting[0].nbytes > self.budget):
                     return
                 r = self._waiting.popleft()
                 self._used += r.nbytes
@@ -330,7 +334,9 @@ class Server:
                     (lf.shape[0],) + tuple(it.dev.verts.shape[1:]), dtype=torch.float32,
                     device=self.device)) for (lf, gv), it in zip(outs, take)]
             b = BatchedLoss([it.dev for it in take], mode=mode, weights=weights, grad=any_grad,
-                            stream=stream, outputs=outs, async_plan=True)
+                            stream=stream, outputs=outs, async_plan=True,
+                            spare=max(0, self.budget - self._used - self._extra))
+            self._extra += b.extra_bytes
             b.run()
             self.host_launch_s.append(time.perf_counter() - t_host)
             done = torch.cuda.Event()
@@ -360,6 +366,7 @@ class Server:
                 if r.left == 0:
                     self._finalize(r, b.stream, status)
             self._busy[s_idx] = None
+            self._extra -= b.extra_bytes
             progressed = True
         return progressed
 
@@ -415,6 +422,7 @@ class Server:
             if busy is not None:
                 for it in busy[2]:
                     reqs[id(it.req)] = it.req
+                self._extra -= busy[0].extra_bytes
                 self._busy[s_idx] = None
         for it in self._admitted:
             reqs[id(it.req)] = it.req

@@ -5,6 +5,7 @@ import ctypes
 import pytest
 import torch
 
+import oracle
 import parity
 import workloads as W
 from paper_2204_03139_gb300 import _lib
@@ -79,3 +80,27 @@ def test_plans_on_the_workspace_of_a_larger_mesh(inputs, small, staged):
     assert parity.rel_l2(b.grad_verts[0].cpu(), grads.cpu()) < 1e-6
     # without room for the other regions either it is refused as before
     assert L.dc_batch_plan(b.frames, b.n_frames, 0, _ptr(small), 1 << 20, st) == _lib.DC_ENOSPC
+
+
+def test_server_admits_a_face_heavy_request_by_its_least_workspace():
+    """A budget that holds the request without the pruned search's regions: it is served, and the
+    running batch's bytes are given back."""
+    from paper_2204_03139_gb300.serve import Server, _frames_of, request_bytes
+
+    tr = parity.nudged(W.lift_trajectory(78, 197, T, N, M, name="r"))
+    fr = _frames_of(tr)
+    L = _lib.lib()
+    least, full = (f(fr, tr.T) for f in (L.dc_batch_workspace_least, L.dc_batch_workspace_size))
+    assert least < full
+    need = request_bytes(tr)
+    res = []
+    for budget in (need + 1024, need + 2 * (full - least)):
+        srv = Server(DEV, hbm_budget=budget)
+        res.append(srv.submit(tr).result(timeout=120))
+        srv.close()
+        assert srv._used == 0 and srv._extra == 0
+    ref = oracle.loss_traj(tr)
+    for r in res:
+        parity.check_loss(r.loss_frames, ref["loss_frames"])
+        parity.check_grad(r.grad_verts, ref["grad_verts"])
+    assert (res[0].loss_frames == res[1].loss_frames).all()
