@@ -109,23 +109,36 @@ struct KeyBox {
     float x, y, z, inv;
 };
 
-__device__ __forceinline__ unsigned point_key(const unsigned short* t, const KeyBox& b, float x, float y,
-                                              float z) {
+// cell of a point: x | y << 8 | z << 16
+__device__ __forceinline__ unsigned grid_cell(const KeyBox& b, float x, float y, float z) {
     constexpr float TOP = (float)((1 << KEY_AXIS_BITS) - 1);
     // points outside the grid (and NaN) take the nearest cell: keys only order the points
     const unsigned ix = (unsigned)fminf(fmaxf((x - b.x) * b.inv, 0.0f), TOP);
     const unsigned iy = (unsigned)fminf(fmaxf((y - b.y) * b.inv, 0.0f), TOP);
     const unsigned iz = (unsigned)fminf(fmaxf((z - b.z) * b.inv, 0.0f), TOP);
-    return hilbert_key(t, ix, iy, iz);
+    return ix | iy << KEY_AXIS_BITS | iz << (2 * KEY_AXIS_BITS);
+}
+
+__device__ __forceinline__ unsigned point_key(const unsigned short* t, const KeyBox& b, float x, float y,
+                                              float z) {
+    constexpr unsigned MASK = (1u << KEY_AXIS_BITS) - 1;
+    const unsigned c = grid_cell(b, x, y, z);
+    return hilbert_key(t, c & MASK, (c >> KEY_AXIS_BITS) & MASK, c >> (2 * KEY_AXIS_BITS));
 }
 
 // The key grid of a frame, from 128 points of each side: per axis, the medians of the lows and
 // of the highs of 32 groups of 8 points, widened by 15% of their distance (the median low of 8
 // uniform values is at 8% of their range). A few far outliers, which would squeeze the cloud
 // into a few cells of their box, do not move the medians. Both sides of a frame compute the same
-// grid from the same points. Called by the whole block; box_sample reads the points, so that
-// other work can be put between their loads and key_box.
+// grid from the same points, so that a query's key finds a block near it on the other side. Where
+// the sides are unlike (apart, or of very different sizes: their own medians differ by more than
+// half the smaller one's extent), that grid may put a whole side into a few cells, unsorted, and
+// nothing could be pruned there: a side whose sample lies in clearly fewer of its coarse cells
+// than of those of the grid of its own medians takes the latter. 8 frames of 10 000 points a side, 10 extents apart: 1390 -> 205 us; one
+// side 1000 times smaller: 880 -> 210 us. Called by the whole block; box_sample reads the points,
+// so that other work can be put between their loads and key_box; s_p is scratch.
 constexpr int BOX_THREADS = 256;
+static_assert(PREP_WARPS >= 12, "a warp per median");
 struct BoxSample {
     float p[3];
 };
@@ -141,15 +154,58 @@ __device__ __forceinline__ BoxSample box_sample(const float* __restrict__ P, int
     }
     return b;
 }
-__device__ KeyBox key_box(const BoxSample& b) {
+// the grid over the box of lows med[0..2] and negated highs med[3..5]
+__device__ __forceinline__ KeyBox grid_of(const float* med) {
+    float lo[3], ext = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float a = med[k], h = -med[3 + k];
+        const float d = fmaxf(h - a, 0.0f);
+        lo[k] = fabsf(a) <= COORD_MAX ? a - 0.15f * d : 0.0f;
+        ext = fmaxf(ext, 1.3f * d);
+    }
+    KeyBox r{lo[0], lo[1], lo[2], 0.0f};
+    r.inv = ext > 1e-30f && ext < 1e30f ? (float)(1 << KEY_AXIS_BITS) / ext : 0.0f;
+    return r;
+}
+
+// The grid of a side unlike the other (see key_box). Called by the whole block; out of line, so that
+// the preparation keeps its registers.
+__device__ __noinline__ KeyBox unlike_grid(BoxSample b, int side, KeyBox both, KeyBox own,
+                                                unsigned* s_cell) {
+    // points of the side's sample in the coarse cell (of 8 per axis) of one before them, in either
+    // grid: at random in space about 15 of 128, on a surface 70, on a line 120
+    constexpr unsigned COARSE = 0xE0E0E0u;
+    constexpr int CLEARLY = 32;
+    static_assert(KEY_AXIS_BITS == 8, "top three bits of each axis");
+    constexpr int HALF = BOX_THREADS / 2;
+    const int t = (int)threadIdx.x - side * HALF;
+    const bool mine = t >= 0 && t < HALF;
+    if (mine) {
+        s_cell[t] = grid_cell(both, b.p[0], b.p[1], b.p[2]) & COARSE;
+        s_cell[HALF + t] = grid_cell(own, b.p[0], b.p[1], b.p[2]) & COARSE;
+    }
+    __syncthreads();
+    bool met[2] = {false, false};
+    if (mine)
+        for (int j = 0; j < t; ++j) {
+            met[0] |= s_cell[j] == s_cell[t];
+            met[1] |= s_cell[HALF + j] == s_cell[HALF + t];
+        }
+    const int in_both = __syncthreads_count(met[0]), in_own = __syncthreads_count(met[1]);
+    return in_own + CLEARLY <= in_both ? own : both;
+}
+
+__device__ KeyBox key_box(const BoxSample& b, int side, float (*s_p)[BOX_THREADS]) {
     __shared__ float s_low[6][32];  // lows, then negated highs, of every group
-    __shared__ float s_med[6];
+    __shared__ float s_med[3][6];   // medians: of both sides' groups, of each side's
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < BOX_THREADS) {
         float v[6];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const bool ok = coord_ok(b.p[k]);
+            s_p[k][tid] = b.p[k];
             v[k] = ok ? b.p[k] : INFINITY;
             v[3 + k] = ok ? -b.p[k] : INFINITY;
         }
@@ -170,20 +226,38 @@ __device__ KeyBox key_box(const BoxSample& b) {
             const float u = __shfl_sync(0xffffffffu, v, j);
             rank += u < v || (u == v && j < lane) ? 1 : 0;
         }
-        if (rank == 16) s_med[warp] = v;
+        if (rank == 16) s_med[0][warp] = v;
+    } else if (warp < 12) {
+        // of a side's 16 groups: rank 8. Here a group is every 16th point of the sample, so that it
+        // spans the cloud also where neighbours follow each other (the rows of a mesh).
+        const int k = warp - 6 < 3 ? warp - 6 : warp - 9;
+        const float sign = warp - 6 < 3 ? 1.0f : -1.0f;
+        float v = INFINITY;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float p = s_p[k][(lane >> 4) * (BOX_THREADS / 2) + 16 * j + (lane & 15)];
+            if (coord_ok(p)) v = fminf(v, sign * p);
+        }
+        int rank = 0;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const float u = __shfl_sync(0xffffffffu, v, (lane & 16) + j);
+            rank += u < v || (u == v && j < (lane & 15)) ? 1 : 0;
+        }
+        if (rank == 8) s_med[1 + (lane >> 4)][warp - 6] = v;
     }
     __syncthreads();
-    float lo[3], ext = 0.0f;
+    float ext[2] = {0.0f, 0.0f}, off = 0.0f;  // of the sides; how far their medians differ
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float a = s_med[k], h = -s_med[3 + k];
-        const float d = fmaxf(h - a, 0.0f);
-        lo[k] = fabsf(a) <= COORD_MAX ? a - 0.15f * d : 0.0f;
-        ext = fmaxf(ext, 1.3f * d);
-    }
-    KeyBox r{lo[0], lo[1], lo[2], 0.0f};
-    r.inv = ext > 1e-30f && ext < 1e30f ? (float)(1 << KEY_AXIS_BITS) / ext : 0.0f;
-    return r;
+    for (int k = 0; k < 6; ++k) off = fmaxf(off, fabsf(s_med[1][k] - s_med[2][k]));
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            ext[q] = fmaxf(ext[q], -s_med[1 + q][3 + k] - s_med[1 + q][k]);
+    const KeyBox both = grid_of(s_med[0]);
+    if (off <= 0.5f * fminf(ext[0], ext[1])) return both;
+    return unlike_grid(b, side, both, grid_of(s_med[1 + side]), reinterpret_cast<unsigned*>(s_p));
 }
 
 // ---------------------------------------------------------------------------------------
@@ -318,8 +392,14 @@ template <int S>
 __global__ void __launch_bounds__(PREP_THREADS, 2)
     k_tree_prep(UniformArgs a, Ws w, int uniform, int n_frames, int rows, int cdf_shared) {
     __shared__ __align__(16) unsigned short s_tab[24 * 64];
-    for (int i = threadIdx.x; i < 24 * 32; i += PREP_THREADS)
-        reinterpret_cast<unsigned*>(s_tab)[i] = reinterpret_cast<const unsigned*>(c_hilbert.v)[i];
+    constexpr int TAB_WORDS = (24 * 32 + PREP_THREADS - 1) / PREP_THREADS;
+    static_assert(sizeof(s_tab) >= 3 * BOX_THREADS * sizeof(float), "key_box's scratch");
+    unsigned tab[TAB_WORDS];
+#pragma unroll
+    for (int h = 0; h < TAB_WORDS; ++h)
+        tab[h] = threadIdx.x + h * PREP_THREADS < 24 * 32
+                     ? reinterpret_cast<const unsigned*>(c_hilbert.v)[threadIdx.x + h * PREP_THREADS]
+                     : 0u;
     pdl_wait();
     cg::cluster_group cl = cg::this_cluster();
     auto meet = [&]() {
@@ -429,7 +509,15 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
         }
         if (bad) set_status(&s_err, DC_EINVAL);
     }
-    const KeyBox box = key_box(sample);
+    // the Hilbert table's memory is key_box's scratch first: 3 KB more would cost two CTAs on meshes of
+    // 19 600 faces (78 KB of areas each) the step from 92 to 60 KB of L1, 430 -> 490 us for 100 frames
+    const KeyBox box = key_box(sample, side, reinterpret_cast<float(*)[BOX_THREADS]>(s_tab));
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < TAB_WORDS; ++h)
+        if (tid + h * PREP_THREADS < 24 * 32)
+            reinterpret_cast<unsigned*>(s_tab)[tid + h * PREP_THREADS] = tab[h];
+    __syncthreads();
     if (sampled) {
         meet();  // all areas are in place
         // a CDF too large for shared memory lives in the frame's global slot, scanned by CTA 0

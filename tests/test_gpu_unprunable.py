@@ -25,6 +25,16 @@ def clouds(case):
         a[:, N // 10:], b[:, N // 10:] = 0.0, 0.0
     elif case == "tied":  # so far apart that all distances round to the same value
         a += 1e8
+    elif case == "apart":
+        a += 10.0
+    elif case == "apart_along_x":
+        a[..., 0] += 10.0
+    elif case == "small_beside_large":
+        a = 0.4 + 1e-3 * a
+    elif case == "one_target":
+        b[:] = 0.3
+    elif case == "one_sim_point":
+        a[:] = 0.3
     return (torch.from_numpy(x.astype(np.float32)).to(DEV) for x in (a, b))
 
 
@@ -42,7 +52,8 @@ def _time(fn):
 
 
 @pytest.mark.parametrize("mode", [0, 1])
-@pytest.mark.parametrize("case", ["coincident", "mostly_coincident", "tied"])
+@pytest.mark.parametrize("case", ["coincident", "mostly_coincident", "tied", "apart", "apart_along_x",
+                                  "small_beside_large", "one_target", "one_sim_point"])
 def test_results_and_time_against_the_direct_engine(case, mode):
     a, b = clouds(case)
     out, ms = [], []
