@@ -10,7 +10,9 @@ dc_loss_traj call per frame, no graph.
 """
 from __future__ import annotations
 
+import collections
 import ctypes
+import threading
 from dataclasses import dataclass
 
 import numpy as np
@@ -62,6 +64,27 @@ FRAME_DTYPE = np.dtype([("verts", "u8"), ("faces", "u8"), ("face_mask", "u8"), (
 assert FRAME_DTYPE.itemsize == ctypes.sizeof(_lib.dc_frame)
 for _name, _ in _lib.dc_frame._fields_:
     assert FRAME_DTYPE.fields[_name][1] == getattr(_lib.dc_frame, _name).offset
+
+
+# Per stream, the pinned staging of asynchronous plans with the event that follows the upload. The
+# library queues the upload, so torch's pinned allocator does not know that the stream still reads
+# the staging and would give the block of a dropped object to the next allocation. A stream's
+# uploads complete in order; completed ones are let go at its next plan. (A copy of torch's own from
+# the staging, which tells its allocator, costs 48 us of host time per plan instead of 24.)
+_uploads: dict = {}
+_uploads_lock = threading.Lock()
+
+
+def _keep_until_uploaded(staging, stream):
+    if torch.cuda.is_current_stream_capturing():
+        return  # every replay reads the staging: the captured plan's object has to live as long
+    done = torch.cuda.Event()
+    done.record(stream)
+    with _uploads_lock:
+        queue = _uploads.setdefault((stream.device_index, stream.cuda_stream), collections.deque())
+        while queue and queue[0][0].query():
+            queue.popleft()
+        queue.append((done, staging))
 
 
 class BatchedLoss:
@@ -181,11 +204,7 @@ class BatchedLoss:
                                               ctypes.c_void_p(self.ws.data_ptr()), nb,
                                               ctypes.c_void_p(self._staging.data_ptr()), sb,
                                               ctypes.c_void_p(self.stream.cuda_stream)))
-            # The library queued the upload, so torch's pinned allocator does not know that the
-            # stream still reads the staging; a copy of torch's own from it (into the total,
-            # which a run overwrites) tells it. The block then goes to nobody else before the
-            # upload has completed, also when this object is dropped right after run().
-            self.total.view(torch.uint8).copy_(self._staging[:4], non_blocking=True)
+            _keep_until_uploaded(self._staging, self.stream)
         else:
             _lib._check(L.dc_batch_plan(self.frames, nfr, mode,
                                         ctypes.c_void_p(self.ws.data_ptr()), nb,
