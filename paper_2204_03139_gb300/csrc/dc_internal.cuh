@@ -190,7 +190,8 @@ struct WsHeader {
     int tc_fallback;  // rows whose keys certified no candidate set (scanned in full)
     int tc_next;      // next unit to take, when the pass hands out whole units on demand
     int tree_n;       // pruned search: queued queries
-    int pad[45];
+    int tree_wide;    // and wide tiles met so far
+    int pad[44];
 };
 
 // Byte offsets of every region of a workspace (computed on the host).

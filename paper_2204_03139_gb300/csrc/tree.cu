@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
                 h->tc_fallback = 0;
                 h->tc_next = 0;
                 h->tree_n = 0;
+                h->tree_wide = 0;
             }
         }
     }
@@ -860,6 +861,10 @@ constexpr int OUTLIER_LOG2 = 5;
 // 32 of them, 64-point boxes in all.
 constexpr int WIDE_BOX2 = 16;
 constexpr int WIDE_BOX1 = 40;
+// Tiles that are wide or have this many outliers are rare in ordinary clouds. Beyond one in
+// FEW_WIDE of all tiles (and FEW_WIDE in all) each is looked at for walking as a whole.
+constexpr int MANY_OUTLIERS = 8;
+constexpr int FEW_WIDE = 16;
 // Boxes of 64 points on their way to a warp: their eight boxes of 8 and their points are copied
 // to shared memory while the ones before are searched.
 #ifndef DC_TREE_STAGES
@@ -977,6 +982,80 @@ __device__ __forceinline__ TreeCols tree_cols(const Ws& w, const FrameDesc* fr, 
     return C;
 }
 
+// A tile that meets most boxes, a lane per query (`own`: its bound). First better bounds: every
+// query's distances to the points of the box of 64 nearest to it in the box of 512 nearest to it.
+// If the queries then still need, each by itself, DENSE_SHARE of the boxes of 64 on average (up to
+// 64 of them are tested; at exactly the bound lie ties, which do not count), as where all points are
+// about equally far away or a cloud has too many scales to be sorted, nothing can be pruned, and the
+// tile is walked to the end (done): every box is tested for all of it, a block that any query needs
+// is evaluated by all, its points loaded once for the warp. Where all tiles are like that this is
+// brute force, and a warp per query took up to seven times as long (8 frames of 10 000 points around
+// a sphere's centre against as many on it: 4650 us, now 930).
+struct TileWalk {
+    float md;  // the minimum (the bound, if not done), its lowest index and place
+    int nn, at;
+    bool done;
+};
+constexpr float DENSE_SHARE = 0.25f;
+__device__ __noinline__ TileWalk walk_tile(TreeCols C, const float* qb, float own, bool valid) {
+    const float3 q = make_float3(__ldg(qb), __ldg(qb + 8), __ldg(qb + 16));
+    const float2 nx = make_float2(-q.x, -q.x), ny = make_float2(-q.y, -q.y),
+                 nz = make_float2(-q.z, -q.z);
+    auto bound = [&](const float4* box, int i) {
+        return box_bound(q, q, __ldg(box + 2 * i), __ldg(box + 2 * i + 1));
+    };
+    // this lane's nearest of the boxes [a, b), the first among equals
+    auto nearest = [&](const float4* box, int a, int b) {
+        float l = INFINITY;
+        int at = a;
+        for (int k = a; k < b; ++k) {
+            const float t = bound(box, k);
+            if (t < l) l = t, at = k;
+        }
+        return at;
+    };
+    const int b2 = nearest(C.box2, 0, C.nb2);
+    const int b1 = nearest(C.box1, 8 * b2, min(8 * b2 + 8, C.nb1));
+    for (int b = 8 * b1; b < min(8 * b1 + 8, C.nb); ++b) {
+        float2 d[4];
+        block_dist(C.pts + 8LL * b, nx, ny, nz, d);
+        own = fminf(own, block_min(d));
+    }
+    __syncwarp();
+    const int step = (C.nb1 + 63) / 64;
+    int need = 0, boxes = 0;
+    for (int b = 0; b < C.nb1; b += step, ++boxes) need += bound(C.box1, b) < own ? 1 : 0;
+    const int all = __reduce_add_sync(0xffffffffu, valid ? need : 0);
+    const int queries = __popc(__ballot_sync(0xffffffffu, valid));
+    TileWalk r{own, 0x7fffffff, 0, (float)all > DENSE_SHARE * (float)(boxes * queries)};
+    if (!r.done) return r;
+    if (!valid) r.md = -1.0f;  // needs nothing
+    auto meets = [&](const float4* box, int i) {
+        return __any_sync(0xffffffffu, bound(box, i) <= r.md);
+    };
+    for (int i2 = 0; i2 < C.nb2; ++i2) {
+        if (!meets(C.box2, i2)) continue;
+        for (int i1 = 8 * i2; i1 < min(8 * i2 + 8, C.nb1); ++i1) {
+            if (!meets(C.box1, i1)) continue;
+#pragma unroll 2
+            for (int b = 8 * i1; b < min(8 * i1 + 8, C.nb); ++b) {
+                float2 d[4];
+                block_dist(C.pts + 8LL * b, nx, ny, nz, d);
+                if (block_min(d) > r.md) continue;
+                const float* id = reinterpret_cast<const float*>(C.pts + 8LL * b) + 24;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float v = j & 1 ? d[j >> 1].y : d[j >> 1].x;
+                    if (!(v <= r.md)) continue;  // (NaN: no distance)
+                    const int i = __float_as_int(__ldg(id + j));
+                    if (v < r.md || i < r.nn) r.md = v, r.nn = i, r.at = 8 * b + j;
+                }
+            }
+        }
+    }
+    return r;
+}
+
 // Every warp takes 32 consecutive queries of one side of one frame in sorted order, so they lie
 // close together and mostly need the same boxes.
 //   - Starting bounds: the block at each query's own key among the other side's keys.
@@ -1035,15 +1114,15 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     const bool valid = pos0 + lane < n;
     float own;  // its bound
     bool act;
+    const int own_pos = min(pos0 + lane, n - 1);
+    const float* const qb = w.tpts + 4LL * (gt - pos0) + 32LL * (own_pos >> 3) + (own_pos & 7);
     {
-        const int pos = min(pos0 + lane, n - 1);
-        const float* qb = w.tpts + 4LL * (gt - pos0) + 32LL * (pos >> 3) + (pos & 7);
         const float qx = __ldg(qb), qy = __ldg(qb + 8), qz = __ldg(qb + 16);
         // Starting bound: the last block whose first key is not above the query's own. The warp
         // narrows the tile's first key down to 32 blocks, 32 probes per step; each query then
         // looks among these (their keys lie close together; beyond the last one it takes that).
         const unsigned* kc = w.tkb + (side ? fr->row0 : (long long)rows + fr->col0) / 8;
-        const unsigned key = __ldg(w.tkey + (gt - pos0) + pos);
+        const unsigned key = __ldg(w.tkey + (gt - pos0) + own_pos);
         const unsigned key0 = __shfl_sync(0xffffffffu, key, 0);
         int lo = 0;
         for (int len = C.nb; len > 32;) {
@@ -1151,8 +1230,20 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
         }
         __syncwarp();
     }
+    bool done = false;  // by walk_tile, its indices and places in sw.hit (free then)
+    if (wide || __popc(__ballot_sync(0xffffffffu, valid && !act)) >= MANY_OUTLIERS) {
+        int met = 0;
+        if (lane == 0) met = atomicAdd(&w.hdr->tree_wide, 1);
+        met = __shfl_sync(0xffffffffu, met, 0);
+        if (met >= max(FEW_WIDE, (int)gridDim.x / FEW_WIDE)) {
+            const TileWalk r = walk_tile(C, qb, own, valid);
+            own = r.md;
+            done = r.done;
+            if (done) sw.hit[lane] = r.nn, sw.hit[32 + lane] = r.at;
+        }
+    }
     // their blocks
-    if (!wide) {
+    if (!wide && !done) {
         auto stage = [&](int h) {
             if (h < hits) {
                 TreeStage& st = sw.stage[h & (STAGES - 1)];
@@ -1209,7 +1300,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     float md = own;
     int nn = 0x7fffffff, at = 0;
     const unsigned tied = __ballot_sync(0xffffffffu, tie) >> (lane & ~3);
-    const bool alone = valid && (wide || !act || (tied & 0xfu) != 0);
+    const bool alone = valid && !done && (wide || !act || (tied & 0xfu) != 0);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         float v = best[j];
@@ -1240,6 +1331,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
             md = fminf(md, v);
         }
     }
+    if (done) nn = sw.hit[lane], at = sw.hit[32 + lane];  // (own is the minimum)
     // the pair's gradient, added to the sim point's (the query's own, or its neighbour's for a
     // target query), 16 bytes at once
     const float gs = grad_scale(fr, side, bidir);

@@ -31,6 +31,17 @@ def clouds(case):
         a[..., 0] += 10.0
     elif case == "small_beside_large":
         a = 0.4 + 1e-3 * a
+    elif case == "sphere_and_centre":  # equidistant, many of the distances exactly
+        b -= 0.5
+        b /= np.linalg.norm(b, axis=2, keepdims=True)
+        a = 1e-4 * (a - 0.5)
+    elif case == "sphere_and_inside":
+        b -= 0.5
+        b /= np.linalg.norm(b, axis=2, keepdims=True)
+        a = 0.3 * (a - 0.5)
+    elif case == "many_scales":  # around the origin, too dense there for the sort's cells
+        a = 10 ** (-6 * rng.random((T, N, 1))) * (a - 0.5)
+        b = 10 ** (-6 * rng.random((T, N, 1))) * (b - 0.5)
     elif case == "one_target":
         b[:] = 0.3
     elif case == "one_sim_point":
@@ -53,7 +64,8 @@ def _time(fn):
 
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("case", ["coincident", "mostly_coincident", "tied", "apart", "apart_along_x",
-                                  "small_beside_large", "one_target", "one_sim_point"])
+                                  "small_beside_large", "one_target", "one_sim_point",
+                                  "sphere_and_centre", "sphere_and_inside", "many_scales"])
 def test_results_and_time_against_the_direct_engine(case, mode):
     a, b = clouds(case)
     out, ms = [], []
@@ -64,3 +76,34 @@ def test_results_and_time_against_the_direct_engine(case, mode):
     for x, y in zip(*out):
         assert x is None and y is None or torch.equal(x, y)
     assert ms[0] < 6 * ms[1]
+
+
+@pytest.mark.parametrize("n,m", [(2600, 2600), (2600, 33), (5000, 3001), (40, 9000)])
+def test_walked_tiles_at_ragged_sizes(n, m):
+    """Gradient too: equidistant clouds of sizes that leave ragged tiles and blocks."""
+    rng = np.random.default_rng(n + m)
+    x = rng.normal(size=(6, m, 3))
+    y = torch.from_numpy((x / np.linalg.norm(x, axis=2, keepdims=True)).astype(np.float32)).to(DEV)
+    v = torch.from_numpy((1e-3 * rng.normal(size=(6, 50, 3))).astype(np.float32)).to(DEV)
+    f = torch.from_numpy(rng.permuted(np.tile(np.arange(50), (90, 1)), axis=1)[:, :3].astype(
+        np.int32)).to(DEV)
+    d = torch.from_numpy(rng.random((6, n, 3)).astype(np.float32)).to(DEV)
+    out = []
+    for shape in (PRUNED, DIRECT):
+        with autotune.tuned(shape):
+            out.append(_lib.dc_loss_traj(v, f, d, y, check=True))
+    for k in ("loss_total", "loss_frames", "nn_ab", "nn_ba"):
+        assert torch.equal(out[0][k], out[1][k])
+    # the gradient in 64 bits, from the library's own samples and neighbours
+    p, face, bary = (x.double() if x.is_floating_point() else x.long()
+                     for x in _lib.dc_sample(v, f, d, check=True))
+    nab, nba = out[0]["nn_ab"].long(), out[0]["nn_ba"].long()
+    ref = torch.zeros(v.shape, dtype=torch.float64, device=DEV)
+    for t in range(v.shape[0]):
+        yt = y[t].double()
+        gx = 2.0 / n * (p[t] - yt[nab[t]])
+        gx.index_add_(0, nba[t], 2.0 / m * (p[t][nba[t]] - yt))
+        ref[t].index_add_(0, f.long()[face[t]].reshape(-1),
+                          (bary[t][:, :, None] * gx[:, None, :]).reshape(-1, 3))
+    for o in out:
+        assert float((o["grad_verts"].double() - ref).norm() / ref.norm()) < 1e-6
