@@ -270,6 +270,10 @@ typedef struct dc_tune {
 } dc_tune;
 
 int dc_tune_set(const dc_tune* tune); /* NULL restores automatic */
+/* The engine (DC_ENGINE_*) of the last forward call on a workspace, or that its batch plan was made
+ * with: dc_tune_set asks for an engine, and a problem that it does not take runs the direct engine.
+ * Waits for `stream`; a negative error code on failure. */
+int dc_ws_engine(const void* ws, dc_stream_t stream);
 int dc_tune_get(dc_tune* tune);
 
 /*

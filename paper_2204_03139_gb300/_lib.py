@@ -84,6 +84,7 @@ def lib() -> ctypes.CDLL:
                 "dc_loss_total": (I, [P, P, I, P, P]),
                 "dc_batch_run": (I, [P, P, P]),
                 "dc_ws_status": (I, [P, P]),
+                "dc_ws_engine": (I, [P, P]),
                 "dc_last_error": (ctypes.c_char_p, []),
                 "dc_launch_count": (ctypes.c_longlong, []),
                 "dc_prof_start": (I, [I]),
@@ -217,6 +218,15 @@ def ws_status(ws: torch.Tensor, stream=None) -> int:
     """Device-side status of the calls issued on `stream` (default: current) with ws."""
     s = _stream(ws.device) if stream is None else stream.cuda_stream
     return int(lib().dc_ws_status(_ptr(ws), s))
+
+
+def ws_engine(ws: torch.Tensor) -> int:
+    """ENGINE_* that the last forward call on the current stream with ws ran (or that its batch
+    plan was made with)."""
+    rc = int(lib().dc_ws_engine(_ptr(ws), _stream(ws.device)))
+    if rc < 0:
+        raise DCError(rc, last_error())
+    return rc
 
 
 def check_ws(ws: torch.Tensor):

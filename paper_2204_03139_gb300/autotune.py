@@ -65,20 +65,27 @@ def _lg(x) -> int:
     return int(math.floor(math.log2(max(1, x))))
 
 
-def bucket(T: int, N: int, M: int, mode: int, device=None) -> str:
-    """Size bucket: device, mode, and powers of two of frames, sim points and targets."""
+# Part of every key: entries of other sets of shapes, which may lack the fastest, are not found.
+_SET = "v2"
+
+
+def bucket(T: int, N: int, M: int, mode: int, device=None, F: int = 0) -> str:
+    """Size bucket: device, mode, and powers of two of frames, sim points, targets and faces."""
     name = torch.cuda.get_device_name(device)
-    return f"{name}|m{mode}|T{_lg(T)}|N{_lg(N)}|M{_lg(M)}"
+    return f"{name}|{_SET}|m{mode}|T{_lg(T)}|N{_lg(N)}|M{_lg(M)}|F{_lg(F)}"
 
 
 def batch_bucket(trajs, mode: int, device=None) -> str:
-    """Size bucket of a batch: frames, mean points per side and total pairs (powers of two)."""
+    """Size bucket of a batch: frames, mean points per side and faces per frame, total pairs
+    (powers of two)."""
     frames = sum(t.T for t in trajs)
     n = sum(int(t.n_off[-1]) for t in trajs) / max(frames, 1)
     m = sum(int(t.m_off[-1]) for t in trajs) / max(frames, 1)
+    faces = sum(t.T * int(t.faces.shape[0]) for t in trajs) / max(frames, 1)
     pairs = sum(t.pairs() for t in trajs)
     name = torch.cuda.get_device_name(device)
-    return f"{name}|batch|m{mode}|F{_lg(frames)}|N{_lg(n)}|M{_lg(m)}|P{_lg(pairs)}"
+    return (f"{name}|{_SET}|batch|m{mode}|T{_lg(frames)}|N{_lg(n)}|M{_lg(m)}|P{_lg(pairs)}"
+            f"|F{_lg(faces)}")
 
 
 def _norm(shape):
@@ -91,9 +98,9 @@ def _norm(shape):
     return (str(e), int(w))
 
 
-def best(T: int, N: int, M: int, mode: int = _lib.BIDIR_MEAN, device=None):
+def best(T: int, N: int, M: int, mode: int = _lib.BIDIR_MEAN, device=None, F: int = 0):
     with _lock:
-        s = _load().get(bucket(T, N, M, mode, device))
+        s = _load().get(bucket(T, N, M, mode, device, F))
     return None if s is None else _norm(s)
 
 
@@ -125,20 +132,28 @@ def _time(fn, dev, reps: int) -> float:
     return a.elapsed_time(b) / reps
 
 
+def _fastest(times, ran):
+    """The fastest shape that ran on its own engine (of all, if none did)."""
+    return min(times, key=lambda sh: (not ran[sh], times[sh]))
+
+
 def tune(verts, faces, draws, targets, mode: int = _lib.BIDIR_MEAN, reps: int = 3,
          save: bool = True, shapes=SHAPES) -> dict:
     """Time dc_loss_traj (forward + gradient) at every shape on these inputs; record and
-    return {"best": shape, "ms": {shape: ms}}."""
+    return {"best": shape, "ms": {shape: ms}}. A shape whose engine does not take the problem
+    (which then runs the direct engine) is not recorded as the best."""
     dev = verts.device
-    T, N, M = verts.shape[0], draws.shape[1], targets.shape[1]
-    times = {}
+    T, N, M, F = verts.shape[0], draws.shape[1], targets.shape[1], faces.shape[0]
+    times, ran = {}, {}
     for sh in shapes:
         with tuned(sh):
             times[sh] = _time(lambda: _lib.dc_loss_traj(verts, faces, draws, targets, mode=mode),
                               dev, reps)
-    s_best = min(times, key=times.get)
+        ws = _lib.workspace(_lib.dc_workspace_size(T, verts.shape[1], F, N, M), dev)
+        ran[sh] = _lib.ws_engine(ws) == _ENGINES[_norm(sh)[0]]
+    s_best = _fastest(times, ran)
     with _lock:
-        _load()[bucket(T, N, M, mode, dev)] = list(s_best)
+        _load()[bucket(T, N, M, mode, dev, F)] = list(s_best)
         if save:
             _save()
     return {"best": s_best, "ms": times}
@@ -151,13 +166,14 @@ def tune_batch(trajs, mode: int = _lib.BIDIR_MEAN, weights=None, grad: bool = Tr
     from .batch import BatchedLoss
 
     dev = trajs[0].verts.device
-    times = {}
+    times, ran = {}, {}
     for sh in shapes:
         with tuned(sh):
             b = BatchedLoss(trajs, mode=mode, weights=weights, grad=grad)
         times[sh] = _time(b.run, dev, reps)
+        ran[sh] = _lib.ws_engine(b.ws) == _ENGINES[_norm(sh)[0]]
         del b
-    s_best = min(times, key=times.get)
+    s_best = _fastest(times, ran)
     with _lock:
         _load()[batch_bucket(trajs, mode, dev)] = list(s_best)
         if save:
@@ -175,7 +191,7 @@ def loss_traj(verts, faces, draws, targets, mode: int = _lib.BIDIR_MEAN, **kw):
     """dc_loss_traj at the tuned shape of its size bucket (tuning the bucket first if it has
     no entry yet)."""
     T, N, M = verts.shape[0], draws.shape[1], targets.shape[1]
-    s = best(T, N, M, mode, verts.device)
+    s = best(T, N, M, mode, verts.device, faces.shape[0])
     if s is None:
         s = tune(verts, faces, draws, targets, mode)["best"]
     with tuned(s):

@@ -581,6 +581,18 @@ int dc_ws_status(const void* ws, dc_stream_t stream) {
     return st;
 }
 
+int dc_ws_engine(const void* ws, dc_stream_t stream) {
+    static_assert(ENGINE_DIRECT == DC_ENGINE_DIRECT && ENGINE_TC == DC_ENGINE_TENSOR &&
+                      ENGINE_TC5 == DC_ENGINE_TCGEN05 && ENGINE_TREE == DC_ENGINE_PRUNED,
+                  "the header holds the public values");
+    if (!ws) return fail(DC_EINVAL, "workspace is NULL");
+    int en = 0;
+    const WsHeader* h = static_cast<const WsHeader*>(ws);
+    cudaError_t e = cudaMemcpyAsync(&en, &h->engine, sizeof(int), cudaMemcpyDeviceToHost, stream);
+    if (!e) e = cudaStreamSynchronize(stream);
+    return e ? cuda_fail(e, "dc_ws_engine") : en;
+}
+
 int dc_area_cdf(const float* verts, const int32_t* faces, const uint8_t* face_mask, int T,
                 int V, int F, float* cdf, void* ws, size_t ws_bytes, dc_stream_t stream) {
     if (T <= 0 || V <= 0 || F <= 0) return fail(DC_EINVAL, "sizes must be positive");

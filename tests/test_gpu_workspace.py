@@ -104,3 +104,22 @@ def test_server_admits_a_face_heavy_request_by_its_least_workspace():
         parity.check_loss(r.loss_frames, ref["loss_frames"])
         parity.check_grad(r.grad_verts, ref["grad_verts"])
     assert (res[0].loss_frames == res[1].loss_frames).all()
+
+
+def test_the_engine_that_ran_is_told_and_tuning_records_no_other(inputs):
+    """A problem whose faces outweigh its points keeps no regions of the pruned search: asked for, it
+    runs the direct engine, which the workspace tells, and the tuner does not record it."""
+    from paper_2204_03139_gb300 import autotune
+
+    d = inputs
+    v, y = d.verts, d.targets.view(T, M, 3)
+    few = d.draws.view(T, N, 3)[:, :500].contiguous()
+    with autotune.tuned(("pruned", 0)):
+        _lib.dc_loss_traj(v, d.faces, few, y)
+    assert _lib.ws_engine(_lib.workspace(1, DEV)) == _lib.ENGINE_DIRECT
+    with autotune.tuned(("pruned", 0)):
+        _lib.dc_chamfer_fwd(few[:1], y[:1])  # points only
+    assert _lib.ws_engine(_lib.workspace(1, DEV)) == _lib.ENGINE_PRUNED
+    shapes = (("pruned", 0), ("direct", 2))
+    r = autotune.tune(v, d.faces, few, y, reps=1, save=False, shapes=shapes)
+    assert r["best"] == ("direct", 2) and set(r["ms"]) == set(shapes)
