@@ -63,7 +63,7 @@ Layout make_layout(const Sizes& s) {
     L.nnba = take(s.cols * 4);
     L.loss = take(s.n_frames * 4);
     L.part = take(s.n_frames * s.slices * 2 * 4);
-    L.frame_err = take(s.n_frames * (s.tree ? 8 : 4));
+    L.frame_err = take(s.n_frames * 4);
     L.fbox = take(s.n_frames * 16);
     L.tsoa = take(6 * s.cols * 4);
     L.tpl = take(3 * s.cols * 4);
@@ -84,6 +84,7 @@ Layout make_layout(const Sizes& s) {
     off = L.tsoa;
     const long long tp = s.tree ? s.rows + s.cols : 0;
     L.y = take(s.tree ? s.cols * 16 : 0);
+    L.tree_err = take(s.tree ? s.n_frames * 8 : 0);
     L.step_frame = take(tp / TREE_STEP * 4);
     L.tkey = take(tp * 4);
     L.tord = take(tp * 8);
@@ -132,6 +133,7 @@ Ws make_ws(void* base, const Layout& L) {
     w.kpart = reinterpret_cast<unsigned*>(p + L.kpart);
     w.tcfb = reinterpret_cast<int*>(p + L.tcfb);
     w.tcfn = reinterpret_cast<int*>(p + L.tcfn);
+    w.tree_err = reinterpret_cast<int*>(p + L.tree_err);
     w.step_frame = reinterpret_cast<int*>(p + L.step_frame);
     w.tkey = reinterpret_cast<unsigned*>(p + L.tkey);
     w.tqueue = reinterpret_cast<int*>(p + L.tord);

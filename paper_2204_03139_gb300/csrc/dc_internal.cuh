@@ -198,7 +198,7 @@ struct WsHeader {
 struct Layout {
     size_t hdr, frames, rowpre, colpre, unit_frame, unit_rb, unit_pre, cdf, x, fw, tsoa, tpl,
         pab, pba, nnab, nnba, loss, part, frame_err, fbox, tc_ufr, tc_urb, tc_upre, tca, tcb,
-        kab, kba, kpart, tcfb, tcfn, step_frame, y, tkey, tord, tpts, tkb, tbox, tbox1, tbox2, frec, tgx, grad4, total;
+        kab, kba, kpart, tcfb, tcfn, tree_err, step_frame, y, tkey, tord, tpts, tkb, tbox, tbox1, tbox2, frec, tgx, grad4, total;
 };
 
 struct Sizes {
@@ -238,8 +238,7 @@ struct Ws {
     int* nnab;         // [rows] fallback neighbour buffers
     int* nnba;         // [cols]
     float* loss;       // [n_frames] fallback loss buffer
-    int* frame_err;    // [n_frames][2] error code of the fused build + area launch, per frame,
-                       // or of the pruned search's preparation, per frame and side
+    int* frame_err;    // [n_frames] error code of the fused build + area launch, per frame
     float* part;       // [n_frames][slices][2] loss partial sums
     float4* fbox;      // [n_frames] (centre x, y, z, scale) of the tensor-core forms
     int* tc_ufr;       // [tc_units] frame of each tensor-core unit
@@ -254,6 +253,7 @@ struct Ws {
                        // certify, each frame's list at its own row (rows + column) range
     int* tcfn;         // [n_frames][2] lengths of those lists (zeroed by the staging)
     // pruned search: sim points then targets, padded as the rows and columns
+    int* tree_err;             // [n_frames][2] error code of the preparation, per frame and side
     int* step_frame;           // [(rows + cols) / TREE_STEP] frame of every step
     unsigned* tkey;            // [rows + cols] curve key of every point; after the preparation
                                // in sorted order

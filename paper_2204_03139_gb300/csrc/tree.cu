@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
         for (int v = r * PREP_THREADS + tid; v < fr.V; v += S * PREP_THREADS)
             w.grad4[fr.v0 + v] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (fr.skip) {  // the same for the whole cluster
-        if (tid == 0 && r == 0) w.frame_err[2 * k + side] = DC_OK;
+        if (tid == 0 && r == 0) w.tree_err[2 * k + side] = DC_OK;
         pdl_trigger();
         return;
     }
@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
         }
     }
     meet();
-    if (tid == 0 && r == 0) w.frame_err[2 * k + side] = s_err;
+    if (tid == 0 && r == 0) w.tree_err[2 * k + side] = s_err;
 
     // ---- boxes: a warp per 512 points, a lane per 8 of them, twice. The w lane of the lower
     // corner of a box of 64 or 512 holds the lowest index in it: a box at exactly a query's minimum
@@ -1088,7 +1088,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
     const int pos0 = gt - (side ? rows + fr->col0 : fr->row0);
     if (pos0 == 0 && lane == 0 && side == 0) {
         // errors of the preparation (both sides; in Eq. 2 the targets are no queries)
-        const int e0 = w.frame_err[2 * k], e1 = w.frame_err[2 * k + 1];
+        const int e0 = w.tree_err[2 * k], e1 = w.tree_err[2 * k + 1];
         if (e0 != DC_OK) set_status(&w.hdr->status, e0);
         if (e1 != DC_OK) set_status(&w.hdr->status, e1);
     }

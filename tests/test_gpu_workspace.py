@@ -123,3 +123,19 @@ def test_the_engine_that_ran_is_told_and_tuning_records_no_other(inputs):
     shapes = (("pruned", 0), ("direct", 2))
     r = autotune.tune(v, d.faces, few, y, reps=1, save=False, shapes=shapes)
     assert r["best"] == ("direct", 2) and set(r["ms"]) == set(shapes)
+
+
+@pytest.mark.parametrize("frames", [1, 32, 33, 57, 300])
+def test_pruned_regions_are_kept_whatever_the_number_of_frames(frames):
+    """Few points per frame, below the line of the default rule: asked for, the pruned search runs."""
+    from paper_2204_03139_gb300 import autotune
+
+    g = torch.Generator(device=DEV).manual_seed(frames)
+    a, b = (torch.rand(frames, n, 3, generator=g, device=DEV) for n in (300, 411))
+    out = []
+    for shape, engine in ((("pruned", 0), _lib.ENGINE_PRUNED), (("direct", 0), _lib.ENGINE_DIRECT)):
+        with autotune.tuned(shape):
+            out.append(_lib.dc_chamfer_fwd(a, b, check=True))
+        assert _lib.ws_engine(_lib.workspace(1, DEV)) == engine
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
