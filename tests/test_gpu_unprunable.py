@@ -94,16 +94,27 @@ def test_walked_tiles_at_ragged_sizes(n, m):
             out.append(_lib.dc_loss_traj(v, f, d, y, check=True))
     for k in ("loss_total", "loss_frames", "nn_ab", "nn_ba"):
         assert torch.equal(out[0][k], out[1][k])
-    # the gradient in 64 bits, from the library's own samples and neighbours
+    # The gradient in 64 bits, from the library's own samples and neighbours. Float32 sums of K terms
+    # in any order are within K u sum |terms|: per vertex, K pairs reach it, each with a few roundings
+    # of its own (difference, factor, weight).
     p, face, bary = (x.double() if x.is_floating_point() else x.long()
                      for x in _lib.dc_sample(v, f, d, check=True))
     nab, nba = out[0]["nn_ab"].long(), out[0]["nn_ba"].long()
-    ref = torch.zeros(v.shape, dtype=torch.float64, device=DEV)
     for t in range(v.shape[0]):
-        yt = y[t].double()
-        gx = 2.0 / n * (p[t] - yt[nab[t]])
-        gx.index_add_(0, nba[t], 2.0 / m * (p[t][nba[t]] - yt))
-        ref[t].index_add_(0, f.long()[face[t]].reshape(-1),
-                          (bary[t][:, :, None] * gx[:, None, :]).reshape(-1, 3))
-    for o in out:
-        assert float((o["grad_verts"].double() - ref).norm() / ref.norm()) < 1e-6
+        yt, corners = y[t].double(), f.long()[face[t]].reshape(-1)
+        ab, ba = 2.0 / n * (p[t] - yt[nab[t]]), 2.0 / m * (p[t][nba[t]] - yt)
+
+        def at_vertices(x):  # [n, c] per point, with its weights
+            w = (bary[t][:, :, None] * x[:, None, :]).reshape(-1, x.shape[1])
+            return torch.zeros(v.shape[1], x.shape[1], dtype=torch.float64,
+                               device=DEV).index_add_(0, corners, w)
+
+        ref = at_vertices(ab.index_add(0, nba[t], ba))
+        size = at_vertices(ab.abs().index_add(0, nba[t], ba.abs()))
+        pairs = torch.ones(n, dtype=torch.float64, device=DEV).index_add_(
+            0, nba[t], torch.ones(m, dtype=torch.float64, device=DEV))
+        reach = torch.zeros(v.shape[1], dtype=torch.float64, device=DEV).index_add_(
+            0, corners, pairs.repeat_interleave(3))
+        for o in out:
+            err = (o["grad_verts"][t].double() - ref).abs()
+            assert bool((err <= 2.0 ** -24 * (reach[:, None] + 8) * size).all())
