@@ -1,9 +1,9 @@
 """Batched loss over many trajectories of uneven sizes (one launch sequence, CUDA graph).
 
 Every frame of every trajectory becomes one dc_frame; dc_batch_plan lays them out in one
-workspace, and dc_batch_run issues the whole sequence -- area CDFs, sampling, ONE persistent
-Chamfer launch whose work split covers all frames, neighbour recovery, losses and the vertex
-gradients -- reading only device memory, so it can be replayed from a CUDA graph.
+workspace, and dc_batch_run issues the whole sequence -- area CDFs, sampling, the
+nearest-neighbour launches over all frames, losses and the vertex gradients -- reading only device
+memory, so it can be replayed from a CUDA graph.
 
 The plain per-frame form (`per_frame_loss`) is the comparison point: the same kernels, one
 dc_loss_traj call per frame, no graph.
@@ -69,22 +69,35 @@ for _name, _ in _lib.dc_frame._fields_:
 # Per stream, the pinned staging of asynchronous plans with the event that follows the upload. The
 # library queues the upload, so torch's pinned allocator does not know that the stream still reads
 # the staging and would give the block of a dropped object to the next allocation. A stream's
-# uploads complete in order; completed ones are let go at its next plan. (A copy of torch's own from
-# the staging, which tells its allocator, costs 48 us of host time per plan instead of 24.)
+# uploads complete in order; at its next plan completed ones are let go, and one of them is used
+# again, so a stream keeps as many as are in flight. (A new block and event per plan cost 17 us of
+# host time more than none; a copy of torch's own from the staging, which tells its allocator, 48.)
 _uploads: dict = {}
 _uploads_lock = threading.Lock()
 
 
-def _keep_until_uploaded(staging, stream):
+def _upload(stream, nbytes, plan):
+    """Call plan(staging) with pinned memory of nbytes, which is kept until what it queued on
+    `stream` (the current one) has completed. Returns the staging."""
     if torch.cuda.is_current_stream_capturing():
-        return  # every replay reads the staging: the captured plan's object has to live as long
-    done = torch.cuda.Event()
-    done.record(stream)
+        # every replay reads the staging: the captured plan's object has to live as long
+        staging = torch.empty(nbytes, dtype=torch.uint8, pin_memory=True)
+        plan(staging)
+        return staging
+    done = staging = None
     with _uploads_lock:
         queue = _uploads.setdefault((stream.device_index, stream.cuda_stream), collections.deque())
         while queue and queue[0][0].query():
-            queue.popleft()
+            done, staging = queue.popleft()
+    if staging is None or staging.numel() < nbytes:
+        staging = torch.empty(nbytes, dtype=torch.uint8, pin_memory=True)
+    if done is None:
+        done = torch.cuda.Event()
+    plan(staging)
+    done.record(stream)
+    with _uploads_lock:
         queue.append((done, staging))
+    return staging
 
 
 class BatchedLoss:
@@ -199,12 +212,10 @@ class BatchedLoss:
             sb = int(L.dc_batch_plan_bytes(self.frames, nfr, mode))
             if sb == 0:
                 raise _lib.DCError(_lib.DC_EINVAL, "bad batch sizes")
-            self._staging = torch.empty(sb, dtype=torch.uint8, pin_memory=True)
-            _lib._check(L.dc_batch_plan_async(self.frames, nfr, mode,
-                                              ctypes.c_void_p(self.ws.data_ptr()), nb,
-                                              ctypes.c_void_p(self._staging.data_ptr()), sb,
-                                              ctypes.c_void_p(self.stream.cuda_stream)))
-            _keep_until_uploaded(self._staging, self.stream)
+            self._staging = _upload(self.stream, sb, lambda staging: _lib._check(
+                L.dc_batch_plan_async(self.frames, nfr, mode, self.ws.data_ptr(), nb,
+                                      staging.data_ptr(), staging.numel(),
+                                      self.stream.cuda_stream)))
         else:
             _lib._check(L.dc_batch_plan(self.frames, nfr, mode,
                                         ctypes.c_void_p(self.ws.data_ptr()), nb,
