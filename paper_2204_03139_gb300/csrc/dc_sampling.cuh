@@ -194,6 +194,31 @@ __device__ __forceinline__ float bary_point(float w0, float w1, float w2, float 
     return __fmaf_rn(w2, c, __fmaf_rn(w1, b, __fmul_rn(w0, a)));
 }
 
+// The point of the draw (r_f, r1, r2): x = point, q = (face, w0, w1, w2 bits). False, with x = 0
+// and no face, when the face has a vertex index out of range.
+__device__ __forceinline__ bool pick_point(const float* cdf, int F, int V,
+                                           const float* __restrict__ verts,
+                                           const int* __restrict__ faces, float rf, float r1,
+                                           float r2, float4& x, int4& q) {
+    const int f = pick_face(cdf, F, rf);
+    const int i0 = faces[3 * f], i1 = faces[3 * f + 1], i2 = faces[3 * f + 2];
+    if ((unsigned)i0 >= (unsigned)V || (unsigned)i1 >= (unsigned)V ||
+        (unsigned)i2 >= (unsigned)V) {
+        x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        return false;
+    }
+    const float* p0 = verts + 3LL * i0;
+    const float* p1 = verts + 3LL * i1;
+    const float* p2 = verts + 3LL * i2;
+    float w0, w1, w2;
+    bary_weights(r1, r2, w0, w1, w2);
+    x.x = bary_point(w0, w1, w2, p0[0], p1[0], p2[0]);
+    x.y = bary_point(w0, w1, w2, p0[1], p1[1], p2[1]);
+    x.z = bary_point(w0, w1, w2, p0[2], p1[2], p2[2]);
+    q = make_int4(f, __float_as_int(w0), __float_as_int(w1), __float_as_int(w2));
+    return true;
+}
+
 // ---- gradient accumulators of 16 bytes ----
 __device__ __forceinline__ void red_add4(float4* p, float x, float y, float z) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z),

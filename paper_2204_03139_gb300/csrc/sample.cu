@@ -378,29 +378,16 @@ __device__ __forceinline__ void sample_row(const Ws& w, const FrameDesc* fr, int
             if (!(rf >= 0.0f && rf <= 1.0f && r1 >= 0.0f && r1 <= 1.0f && r2 >= 0.0f &&
                   r2 <= 1.0f))
                 set_status(&w.hdr->status, DC_EINVAL);
-            const int f = pick_face(cdf, fr->F, rf);
-            const int i0 = fr->faces[3 * f], i1 = fr->faces[3 * f + 1], i2 = fr->faces[3 * f + 2];
-            const int V = fr->V;
-            if ((unsigned)i0 < (unsigned)V && (unsigned)i1 < (unsigned)V &&
-                (unsigned)i2 < (unsigned)V) {
-                const float* p0 = fr->verts + 3LL * i0;
-                const float* p1 = fr->verts + 3LL * i1;
-                const float* p2 = fr->verts + 3LL * i2;
-                float w0, w1, w2;
-                bary_weights(r1, r2, w0, w1, w2);
-                x.x = bary_point(w0, w1, w2, p0[0], p1[0], p2[0]);
-                x.y = bary_point(w0, w1, w2, p0[1], p1[1], p2[1]);
-                x.z = bary_point(w0, w1, w2, p0[2], p1[2], p2[2]);
-                q = make_int4(f, __float_as_int(w0), __float_as_int(w1), __float_as_int(w2));
+            if (pick_point(cdf, fr->F, fr->V, fr->verts, fr->faces, rf, r1, r2, x, q)) {
+                const int f = q.x;
                 if (fr->out_face) fr->out_face[i] = f;
                 if (fr->out_bary) {
-                    fr->out_bary[3LL * i] = w0;
-                    fr->out_bary[3LL * i + 1] = w1;
-                    fr->out_bary[3LL * i + 2] = w2;
+                    fr->out_bary[3LL * i] = __int_as_float(q.y);
+                    fr->out_bary[3LL * i + 1] = __int_as_float(q.z);
+                    fr->out_bary[3LL * i + 2] = __int_as_float(q.w);
                 }
             } else {
                 set_status(&w.hdr->status, DC_EINVAL);
-                x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
             if (fr->out_pts) {
                 fr->out_pts[3LL * i] = x.x;
