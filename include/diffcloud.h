@@ -235,10 +235,14 @@ int dc_batch_run(void* ws, float* loss_total, dc_stream_t stream);
  *   DC_ENGINE_PRUNED -- the points of both clouds sorted along a space-filling curve, with
  *     bounding boxes of runs of 8, 64 and 512 points; a query evaluates the direct form only for
  *     boxes that its minimum so far does not exclude. Clouds of at most 2 097 152 points, and
- *     at most about 1.5 faces per point where DC_ENGINE_AUTO would not take it.
+ *     at most about 1.5 faces per point where DC_ENGINE_AUTO would not take it (else the direct
+ *     engine runs; dc_ws_engine tells). Its time depends on the clouds: where nothing can be
+ *     excluded (all points about equally far away) it is that of all pairs, up to about 5 times
+ *     the direct engine's.
  *     DC_ENGINE_AUTO takes it for calls (and batch plans) of at least 7e7 pairs (Eq. 2: 9.5e7)
- *     plus 9600 per point of the largest side, 250 per point, 600 + F / 8 per face of the largest
- *     mesh of F faces and 10 per face in all (up to 5 times as many in Eq. 2 with over 3 targets per sim point);
+ *     plus 9600 per point of the largest side, 250 per point of every frame's larger side,
+ *     600 + F / 8 per face of the largest mesh of F faces and 10 per face in all (up to 5 times as
+ *     many in Eq. 2 with over 3 targets per sim point);
  *     else the warp-level tensor filter from 1e9 pairs and 5e7 per frame on, and the direct
  *     engine below.
  *   DC_ENGINE_TENSOR -- a tensor-core filter: the expanded form |p|^2 - 2 p.q + |q|^2 on
@@ -335,8 +339,9 @@ int dc_fp32_fma_rate(int packed, int iters, double* flop_per_s, dc_stream_t stre
  * The next nearest-neighbour launch of an engine with bounded waits (all but the pruned search)
  * in the process never requests the first target chunk of each CTA, so the waits on it give up
  * after 2 s: the call completes, its workspace reports DC_ETIMEOUT (dc_ws_status), and the
- * device stays usable for the next call. While it is pending, calls under DC_ENGINE_AUTO and
- * runs of planned batches take the direct engine instead of the pruned search.
+ * device stays usable for the next call. While it is pending, calls under DC_ENGINE_AUTO take the
+ * engine they would take without the pruned search (the tensor-core filter or the direct engine),
+ * and runs of planned batches the direct engine.
  */
 int dc_test_inject_stall(void);
 

@@ -124,8 +124,12 @@ enum : int {
     ENGINE_TC5 = 3,
     ENGINE_TREE = 4
 };
-constexpr int TREE_STEP = 256;  // queries per CTA of the pruned search (frames start at multiples)
-constexpr int TREE_MAX_POINTS = 1 << 21;  // points per side (index bits beside a key's low bits)
+// padded points per entry of step_frame, and per block of the gradient's scatter (frames start at
+// multiples)
+constexpr int TREE_STEP = 256;
+// Points per side: the counting sort has 2^14 cells for clouds over 65 535 points, 128 points in each
+// on average here; cells of more than 256 stay unsorted inside.
+constexpr int TREE_MAX_POINTS = 1 << 21;
 static_assert(ROW_PAD % TREE_STEP == 0 && COL_PAD % TREE_STEP == 0, "steps lie in one frame");
 __host__ __device__ inline bool keyed(int engine) {
     return engine == ENGINE_TC || engine == ENGINE_TC5;
@@ -184,12 +188,12 @@ struct WsHeader {
     int max_v;        // largest V among frames with a gradient
     int slices;       // epilogue slices per frame
     int warps;        // warps per Chamfer CTA (units of warps * ROWS_PER_WARP sim points)
-    int engine;       // ENGINE_DIRECT, ENGINE_TC or ENGINE_TC5
+    int engine;       // ENGINE_* that ran, or that the plan was made with
     int tc_units;     // tensor-core work units (frame, side, 512 rows)
     int tc_total;     // their chunks of TC_CHUNK columns (live frames only)
     int tc_fallback;  // rows whose keys certified no candidate set (scanned in full)
     int tc_next;      // next unit to take, when the pass hands out whole units on demand
-    int tree_n;       // pruned search: queued queries
+    int tree_n;       // pruned search: queries queued for the single search
     int tree_wide;    // and wide tiles met so far
     int pad[44];
 };
@@ -258,7 +262,7 @@ struct Ws {
     unsigned* tkey;            // [rows + cols] curve key of every point; after the preparation
                                // in sorted order
     float4* y;                 // [cols] targets as given (w lane unused)
-    unsigned long long* tord;  // [rows + cols] cell, low key bits, index in counting-sort order
+    unsigned long long* tord;  // [rows + cols] index << 32 | key << 8 in counting-sort order
     int* tqueue;               // queries searched one at a time (the region of tord)
     float* tpts;               // [rows + cols][4] sorted blocks of 8: x[8] y[8] z[8] index[8]
     unsigned* tkb;             // [(rows + cols) / 8] first key of every block
@@ -335,7 +339,7 @@ struct UniformArgs {
     const float* gframes;  // [T] nullable (backward only): dJ/dL_t directly
     int bwd;               // 1: gradient multipliers g_t = w_t gtotal + gframes[t]
     int T, V, F, N, M, mode, units_per_frame, subs_per_unit, slices, warps;
-    int engine;            // ENGINE_DIRECT, ENGINE_TC or ENGINE_TC5 (calls with a Chamfer)
+    int engine;            // ENGINE_* (calls with a Chamfer)
 };
 
 cudaError_t launch_build_uniform(const UniformArgs& a, const Ws& w, cudaStream_t s);

@@ -42,7 +42,7 @@ struct EpiArgs {
     int flags;     // EPI_RESCAN | EPI_LOSS | EPI_GRAD
     int bidir;
     int use_smem;  // one slice per frame and the V x 3 accumulator fits in shared memory
-    int exact;     // the packed minima hold the neighbour's index itself (all but the direct engine)
+    int exact;     // the packed minima hold the neighbour's index itself (tensor-core filters)
 };
 
 __device__ __forceinline__ float block_sum_fixed(float v, float* s_red) {
@@ -113,7 +113,9 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
     const float* PX = w.tpl + 3LL * col0;  // compact target planes X[Mpad], Y, Z
     const float* PY = PX + fr->Mpad;
     const float* PZ = PY + fr->Mpad;
-    const float* tgt = fr->tgt;  // as given: the exact mode (the pruned search stages no planes)
+    // Targets as given, for the exact mode: a neighbour's three coordinates lie in one or two lines,
+    // in the planes in three (tensor-core filter, 4 frames of 32 768 points: 789 against 796 us).
+    const float* tgt = fr->tgt;
     const int i0 = (int)((long long)N * sl / e.slices);
     const int i1 = (int)((long long)N * (sl + 1) / e.slices);
     const bool exact = e.exact != 0 && rescan;
@@ -146,7 +148,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
                         kahan_add(sab, cab_c, __uint_as_float((unsigned)(pr[r] >> 32)));
                     if (pr[r] == EMPTY || (unsigned)nn >= (unsigned)M)
                         set_status(&w.hdr->status, DC_EDEVICE);
-                    if (fr->nn_ab) fr->nn_ab[ir[r]] = nn;
+                    fr->nn_ab[ir[r]] = nn;
                 }
                 nr[r] = vr[r] && (unsigned)nn < (unsigned)M && q < 3 ? nn : -1;
             }
@@ -221,7 +223,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
             if (valid && q == 0) {
                 if (p != EMPTY && want_loss) kahan_add(sab, cab_c, dmin);
                 if (nn < 0) set_status(&w.hdr->status, DC_EDEVICE);
-                if (fr->nn_ab) fr->nn_ab[i] = nn;
+                if (fr->nn_ab) fr->nn_ab[i] = nn;  // (none: a pruned plan under a stall test)
             }
         } else if (valid) {
             nn = fr->nn_ab[i];
@@ -283,7 +285,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_epilogue(Ws w, EpiA
                             kahan_add(sba, cba_c, __uint_as_float((unsigned)(pr[r] >> 32)));
                         if (pr[r] == EMPTY || (unsigned)nn >= (unsigned)N)
                             set_status(&w.hdr->status, DC_EDEVICE);
-                        if (fr->nn_ba) fr->nn_ba[jr[r]] = nn;
+                        fr->nn_ba[jr[r]] = nn;
                     }
                     nr[r] = vr[r] && (unsigned)nn < (unsigned)N && q < 3 ? nn : -1;
                 }

@@ -512,13 +512,13 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
     }
     // the Hilbert table's memory is key_box's scratch first: 3 KB more would cost two CTAs on meshes of
     // 19 600 faces (78 KB of areas each) the step from 92 to 60 KB of L1, 430 -> 490 us for 100 frames
+    // (key_box has met since it last read the scratch)
     const KeyBox box = key_box(sample, side, reinterpret_cast<float(*)[BOX_THREADS]>(s_tab));
-    __syncthreads();
 #pragma unroll
     for (int h = 0; h < TAB_WORDS; ++h)
         if (tid + h * PREP_THREADS < 24 * 32)
             reinterpret_cast<unsigned*>(s_tab)[tid + h * PREP_THREADS] = tab[h];
-    __syncthreads();
+    if (!sampled) __syncthreads();  // (the areas' meeting follows otherwise)
     if (sampled) {
         meet();  // all areas are in place
         // a CDF too large for shared memory lives in the frame's global slot, scanned by CTA 0
@@ -852,13 +852,11 @@ __global__ void __launch_bounds__(PREP_THREADS, 2)
 // values are known to be the same in all lanes: 4.7% faster than two warps on 64 uneven trajectories
 // (18.0 against 18.9 ms), four warps 5.1% slower.
 constexpr int SEARCH_THREADS = 32;
-#ifndef DC_TREE_MIN_BLOCKS
-#define DC_TREE_MIN_BLOCKS 32
-#endif
+constexpr int SEARCH_CTAS = 32;  // per SM: 64 registers (28 CTAs: 18.5 against 18.0 ms)
 // A query whose starting bound is 2^5 times (as squared distance) that of the tile's others
 constexpr int OUTLIER_LOG2 = 5;
-// A tile whose box meets more boxes than this is searched query by query: 512-point boxes per
-// 32 of them, 64-point boxes in all.
+// A tile whose box meets more boxes than this is searched query by query (or walked as a whole, see
+// walk_tile): 512-point boxes per 32 of them, 64-point boxes in all.
 constexpr int WIDE_BOX2 = 16;
 constexpr int WIDE_BOX1 = 40;
 // Tiles that are wide or have this many outliers are rare in ordinary clouds. Beyond one in
@@ -867,10 +865,7 @@ constexpr int MANY_OUTLIERS = 8;
 constexpr int FEW_WIDE = 16;
 // Boxes of 64 points on their way to a warp: their eight boxes of 8 and their points are copied
 // to shared memory while the ones before are searched.
-#ifndef DC_TREE_STAGES
-#define DC_TREE_STAGES 2
-#endif
-constexpr int STAGES = DC_TREE_STAGES;  // a power of two
+constexpr int STAGES = 2;  // a power of two
 struct TreeStage {
     float4 pts[64];  // eight blocks of x[8] y[8] z[8] index[8]
     float4 box[16];  // (lo, hi) of the eight blocks
@@ -1069,14 +1064,15 @@ __device__ __noinline__ TileWalk walk_tile(TreeCols C, const float* qb, float ow
 //   - Only each lane's minimum and its block are tracked; indices are found there at the end.
 //   - Queries that would widen the walk of the others (outliers: a bound far above theirs), all
 //     queries of a tile that meets too many boxes, and queries that met their minimum in two
-//     blocks (exact ties, whose lowest index must win) are queued for k_tree_single.
+//     blocks (exact ties, whose lowest index must win) are queued for k_tree_single; tiles that
+//     nothing prunes are walked as a whole by walk_tile.
 // Bound by instruction issue and the load pipe: 2650 instructions per tile, of which about 20
 // blocks of 8 evaluated (50 each) and 9 boxes of 64 staged are most; 69% of issue slots, 55% of
 // the load pipe's wavefronts, 2.5 cycles per instruction waiting for memory. 40 frames of 10 000
 // points against as many: 94 us, where evaluating every pair takes 630 us (tensor-core filter)
 // or 943 us (direct form). 64 uneven trajectories: 10.8 ms (one query per lane 11.5 ms and
 // 3.8 ms in k_tree_single, without the gradient's sums), the tensor-core filter 158 ms.
-__global__ void __launch_bounds__(SEARCH_THREADS, DC_TREE_MIN_BLOCKS)
+__global__ void __launch_bounds__(SEARCH_THREADS, SEARCH_CTAS)
     k_tree_search(Ws w, int rows, int bidir) {
     pdl_wait();
     __shared__ TreeWarp s_warp[SEARCH_THREADS / 32];
@@ -1573,6 +1569,7 @@ __global__ void __launch_bounds__(OUT_THREADS) k_tree_out(Ws w, int n_frames, in
 }
 
 int g_prep_smem[64];  // per device: dynamic shared memory the preparation may use
+int g_sms[64];        // and SMs
 
 }  // namespace
 
@@ -1583,7 +1580,9 @@ cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max
     if (dev < 0 || dev >= 64) dev = 0;
     constexpr int STATIC = 7 * 1024;  // room for the static shared memory
     if (g_prep_smem[dev] == 0) {
-        int optin = 0;
+        int optin = 0, sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        g_sms[dev] = sms > 0 ? sms : 1;
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         optin = (optin > 0 ? optin : 99 * 1024) - STATIC;
         for (auto f : {k_tree_prep<1>, k_tree_prep<2>, k_tree_prep<3>, k_tree_prep<4>,
@@ -1598,7 +1597,7 @@ cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max
     // (two per SM), each with at least one point per thread.
     int S = 1;
     for (int q : {2, 3, 4, 6, 8})
-        if (2 * n_frames * q <= 2 * 152 && max_n >= q * PREP_THREADS) S = q;
+        if (n_frames * q <= g_sms[dev] && max_n >= q * PREP_THREADS) S = q;
     // the CDF, later the cells and the refinement's buffers: two CTAs per SM up to 27 000 faces
     size_t smem = CELL_BYTES + REFINE_BYTES;
     const bool cdf_shared = 4 * (size_t)max_f <= (size_t)g_prep_smem[dev];
@@ -1635,7 +1634,7 @@ cudaError_t launch_tree(const UniformArgs* a, const Ws& w, int n_frames, int max
     e = launch_pdl(k_tree_search, total / SEARCH_THREADS, SEARCH_THREADS, 0, s, w, rows, bidir);
     count_launch();
     if (!e) {
-        e = launch_pdl(k_tree_single, std::min(16 * 152, total / SINGLE_THREADS), SINGLE_THREADS, 0,
+        e = launch_pdl(k_tree_single, std::min(16 * g_sms[dev], total / SINGLE_THREADS), SINGLE_THREADS, 0,
                        s, w, rows, bidir);
         count_launch();
     }
