@@ -126,17 +126,25 @@ __device__ __forceinline__ unsigned point_key(const unsigned short* t, const Key
     return hilbert_key(t, c & MASK, (c >> KEY_AXIS_BITS) & MASK, c >> (2 * KEY_AXIS_BITS));
 }
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 // The key grid of a frame, from 128 points of each side: per axis, the medians of the lows and
 // of the highs of 32 groups of 8 points, widened by 15% of their distance (the median low of 8
 // uniform values is at 8% of their range). A few far outliers, which would squeeze the cloud
 // into a few cells of their box, do not move the medians. Both sides of a frame compute the same
 // grid from the same points, so that a query's key finds a block near it on the other side. Where
-// the sides are unlike (apart, or of very different sizes: their own medians differ by more than
-// half the smaller one's extent), that grid may put a whole side into a few cells, unsorted, and
-// nothing could be pruned there: a side whose sample lies in clearly fewer of its coarse cells
-// than of those of the grid of its own medians takes the latter. 8 frames of 10 000 points a side, 10 extents apart: 1390 -> 205 us; one
-// side 1000 times smaller: 880 -> 210 us. Called by the whole block; box_sample reads the points,
-// so that other work can be put between their loads and key_box; s_p is scratch.
+// the sides are unlike (apart, or of very different sizes: their own medians differ by over eight
+// times the extent of the common box, which is then near that of their intersection), that grid may
+// put a whole side into a few cells, unsorted, and nothing could be pruned there: a side whose sample
+// lies in clearly fewer of its coarse cells than of those of the grid of its own medians takes the
+// latter (and its starting bounds are loose then: from the extent itself on, one side of half the
+// other's size took 204 instead of 146 us). 8 frames of 10 000 points a side, 10 extents apart:
+// 1390 -> 190 us; one side 1000 times smaller: 880 -> 200 us. Called by the whole block; box_sample
+// reads the points, so that other work can be put between their loads and key_box; s_p is scratch.
 constexpr int BOX_THREADS = 256;
 static_assert(PREP_WARPS >= 12, "a warp per median");
 struct BoxSample {
@@ -199,6 +207,7 @@ __device__ __noinline__ KeyBox unlike_grid(BoxSample b, int side, KeyBox both, K
 __device__ KeyBox key_box(const BoxSample& b, int side, float (*s_p)[BOX_THREADS]) {
     __shared__ float s_low[6][32];  // lows, then negated highs, of every group
     __shared__ float s_med[3][6];   // medians: of both sides' groups, of each side's
+    __shared__ float s_off[6];      // how far the sides' differ
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < BOX_THREADS) {
         float v[6];
@@ -244,19 +253,21 @@ __device__ KeyBox key_box(const BoxSample& b, int side, float (*s_p)[BOX_THREADS
             const float u = __shfl_sync(0xffffffffu, v, (lane & 16) + j);
             rank += u < v || (u == v && j < (lane & 15)) ? 1 : 0;
         }
-        if (rank == 8) s_med[1 + (lane >> 4)][warp - 6] = v;
+        const unsigned who = __ballot_sync(0xffffffffu, rank == 8);  // a lane of each half
+        const float a = __shfl_sync(0xffffffffu, v, __ffs(who) - 1);
+        const float c = __shfl_sync(0xffffffffu, v, 31 - __clz(who));
+        if (lane == 0) {
+            s_med[1][warp - 6] = a;
+            s_med[2][warp - 6] = c;
+            s_off[warp - 6] = fabsf(a - c);
+        }
     }
     __syncthreads();
-    float ext[2] = {0.0f, 0.0f}, off = 0.0f;  // of the sides; how far their medians differ
-#pragma unroll
-    for (int k = 0; k < 6; ++k) off = fmaxf(off, fabsf(s_med[1][k] - s_med[2][k]));
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-            ext[q] = fmaxf(ext[q], -s_med[1 + q][3 + k] - s_med[1 + q][k]);
     const KeyBox both = grid_of(s_med[0]);
-    if (off <= 0.5f * fminf(ext[0], ext[1])) return both;
+    // inv: cells per 1.3 times the extent; an infinite or undefined difference is above any limit
+    const float off = fmaxf(max3(s_off[0], s_off[1], s_off[2]), max3(s_off[3], s_off[4], s_off[5]));
+    constexpr float LIMIT = 8.0f * (float)(1 << KEY_AXIS_BITS) / 1.3f;
+    if (both.inv > 0.0f && off * both.inv <= LIMIT) return both;
     return unlike_grid(b, side, both, grid_of(s_med[1 + side]), reinterpret_cast<unsigned*>(s_p));
 }
 
@@ -894,12 +905,6 @@ struct TreeCols {
     int nb, nb1, nb2;
 };
 
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
 // minimum and maximum over the warp
 __device__ __forceinline__ float warp_min(float v) {
     float r;
@@ -979,13 +984,14 @@ __device__ __forceinline__ TreeCols tree_cols(const Ws& w, const FrameDesc* fr, 
 
 // A tile that meets most boxes, a lane per query (`own`: its bound). First better bounds: every
 // query's distances to the points of the box of 64 nearest to it in the box of 512 nearest to it.
-// If the queries then still need, each by itself, DENSE_SHARE of the boxes of 64 on average (up to
+// If the queries then still need, each by itself, DENSE_SHARE of the boxes of 8 on average (up to
 // 64 of them are tested; at exactly the bound lie ties, which do not count), as where all points are
 // about equally far away or a cloud has too many scales to be sorted, nothing can be pruned, and the
 // tile is walked to the end (done): every box is tested for all of it, a block that any query needs
 // is evaluated by all, its points loaded once for the warp. Where all tiles are like that this is
 // brute force, and a warp per query took up to seven times as long (8 frames of 10 000 points around
-// a sphere's centre against as many on it: 4650 us, now 930).
+// a sphere's centre against as many on it: 4650 us, now 920). At 0.14 of the boxes (clouds side by
+// side) a warp per query is still faster, 230 against 370 us.
 struct TileWalk {
     float md;  // the minimum (the bound, if not done), its lowest index and place
     int nn, at;
@@ -1017,9 +1023,9 @@ __device__ __noinline__ TileWalk walk_tile(TreeCols C, const float* qb, float ow
         own = fminf(own, block_min(d));
     }
     __syncwarp();
-    const int step = (C.nb1 + 63) / 64;
+    const int step = (C.nb + 63) / 64;
     int need = 0, boxes = 0;
-    for (int b = 0; b < C.nb1; b += step, ++boxes) need += bound(C.box1, b) < own ? 1 : 0;
+    for (int b = 0; b < C.nb; b += step, ++boxes) need += bound(C.box0, b) < own ? 1 : 0;
     const int all = __reduce_add_sync(0xffffffffu, valid ? need : 0);
     const int queries = __popc(__ballot_sync(0xffffffffu, valid));
     TileWalk r{own, 0x7fffffff, 0, (float)all > DENSE_SHARE * (float)(boxes * queries)};
@@ -1380,15 +1386,18 @@ __global__ void __launch_bounds__(SINGLE_THREADS, 16) k_tree_single(Ws w, int ro
         float R = __uint_as_float((unsigned)(*slot >> 32));  // the bound so far
         unsigned md = 0x7f800000u, mi = 0x7fffffffu;  // this lane's minimum and its index
         int mb = 0;                                    // and its block
-        // Exact ties: a box of 512 or 64 whose bound is R itself matters only with a lower index
-        // than the lowest one found at R. (Where points coincide, all boxes tie: 8 frames of 10 000
-        // coincident points took 4970 us without this, 270 us with it.)
-        unsigned found = 0x7fffffffu;
-        auto index = [&]() {
-            found = __reduce_min_sync(0xffffffffu, __uint_as_float(md) == R ? mi : 0x7fffffffu);
-        };
-        auto needs = [&](float bound, float first) {
-            return bound < R || (bound == R && __float_as_uint(first) < found);
+        // The lanes whose box (of 512 or 64; bound l, lowest index `first`) matters. Exact ties: one
+        // whose bound is R itself matters only with a lower index than the lowest one found at R.
+        // (Where points coincide, all boxes tie: 8 frames of 10 000 coincident points took 4970 us
+        // without this, 270 us with it.)
+        auto matter = [&](float l, float first) {
+            unsigned m = __ballot_sync(0xffffffffu, l <= R);
+            if (__any_sync(0xffffffffu, l == R)) {
+                const unsigned found =
+                    __reduce_min_sync(0xffffffffu, __uint_as_float(md) == R ? mi : 0x7fffffffu);
+                m = __ballot_sync(0xffffffffu, l < R || (l == R && __float_as_uint(first) < found));
+            }
+            return m;
         };
         // this lane's point of block b
         auto point = [&](int b) {
@@ -1408,7 +1417,7 @@ __global__ void __launch_bounds__(SINGLE_THREADS, 16) k_tree_single(Ws w, int ro
                 first = lo.w;
                 lb = box_bound(q, q, lo, __ldg(C.box2 + 2 * i2 + 1));
             }
-            unsigned m2 = __ballot_sync(0xffffffffu, needs(lb, first));
+            unsigned m2 = matter(lb, first);
             if (s == 0 && __popc(m2) > 2) {
                 // a loose bound: the points of the nearest box of 64 in the nearest box of 512
                 const unsigned near2 = __reduce_min_sync(0xffffffffu, __float_as_uint(lb));
@@ -1424,23 +1433,22 @@ __global__ void __launch_bounds__(SINGLE_THREADS, 16) k_tree_single(Ws w, int ro
                 for (int h = 0; h < 2; ++h)
                     if (8 * n1 + 4 * h + grp < C.nb) point(8 * n1 + 4 * h + grp);
                 R = fminf(R, __uint_as_float(__reduce_min_sync(0xffffffffu, md)));
-                index();
-                m2 = __ballot_sync(0xffffffffu, needs(lb, first));
+                m2 = matter(lb, first);
             }
             while (m2) {
                 const int t2 = take4(m2, grp);
                 const int i1 = (s + t2) * 8 + sub;
-                bool hit = false;
+                float l1 = INFINITY, first1 = 0.f;
                 if (t2 >= 0 && i1 < C.nb1) {
                     const float4 lo = __ldg(C.box1 + 2 * i1);
-                    hit = needs(box_bound(q, q, lo, __ldg(C.box1 + 2 * i1 + 1)), lo.w);
+                    first1 = lo.w;
+                    l1 = box_bound(q, q, lo, __ldg(C.box1 + 2 * i1 + 1));
                 }
-                unsigned m1 = __ballot_sync(0xffffffffu, hit);
-                const bool any = m1 != 0;
+                unsigned m1 = matter(l1, first1);
                 while (m1) {
                     const int t1 = take4(m1, grp);
                     const int i0 = __shfl_sync(0xffffffffu, i1, t1 & 31) * 8 + sub;
-                    hit = false;
+                    bool hit = false;
                     if (t1 >= 0 && i0 < C.nb)
                         hit = box_bound(q, q, __ldg(C.box0 + 2 * i0), __ldg(C.box0 + 2 * i0 + 1)) <= R;
                     unsigned m0 = __ballot_sync(0xffffffffu, hit);
@@ -1451,7 +1459,6 @@ __global__ void __launch_bounds__(SINGLE_THREADS, 16) k_tree_single(Ws w, int ro
                     }
                     R = fminf(R, __uint_as_float(__reduce_min_sync(0xffffffffu, md)));
                 }
-                if (any) index();
             }
         }
         const unsigned dm = __reduce_min_sync(0xffffffffu, md);
