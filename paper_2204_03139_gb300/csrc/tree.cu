@@ -393,7 +393,7 @@ __device__ __forceinline__ int cell_get(const int* h, bool packed, int c) {
 //      (x[8] y[8] z[8] index[8], one 128-byte line)
 //   5. bounding boxes of 8, 64 and 512 consecutive points
 // Bound by latency: chains of dependent gathers (face pick, corners) and one block-wide meeting
-// per phase. 40 frames of 10 000 points against as many: 61 us at 36% of the load pipe, its warps
+// per phase. 40 frames of 10 000 points against as many: 62 us at 37% of the load pipe, its warps
 // waiting 5.3 cycles per instruction for memory and 3.6 at barriers. One kernel for all phases
 // keeps the counters and the draws' points on chip; clusters of 3 instead of 2 for those 80 sides
 // (240 CTAs instead of 160) 210 -> 198 us per call. 64 uneven trajectories, 1.14e8 points:
@@ -1075,8 +1075,8 @@ __device__ __noinline__ TileWalk walk_tile(TreeCols C, const float* qb, float ow
 // Bound by instruction issue and the load pipe: 2650 instructions per tile, of which about 20
 // blocks of 8 evaluated (50 each) and 9 boxes of 64 staged are most; 69% of issue slots, 55% of
 // the load pipe's wavefronts, 2.5 cycles per instruction waiting for memory. 40 frames of 10 000
-// points against as many: 94 us, where evaluating every pair takes 630 us (tensor-core filter)
-// or 943 us (direct form). 64 uneven trajectories: 10.8 ms (one query per lane 11.5 ms and
+// points against as many: 90 us, where evaluating every pair takes 630 us (tensor-core filter)
+// or 943 us (direct form). 64 uneven trajectories: 10.9 ms (one query per lane 11.5 ms and
 // 3.8 ms in k_tree_single, without the gradient's sums), the tensor-core filter 158 ms.
 __global__ void __launch_bounds__(SEARCH_THREADS, SEARCH_CTAS)
     k_tree_search(Ws w, int rows, int bidir) {
@@ -1367,7 +1367,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, SEARCH_CTAS)
 // lane one point of four blocks of 8. Bound by latency (three levels of dependent loads, 12.6
 // cycles per instruction), so 64 warps per SM at 32 registers, although that spills: with 42 or
 // 51 registers (48 and 40 warps) the 100-frame call of 32 768 points takes 1770 and 1784 us
-// instead of 1755. 64 uneven trajectories 0.96 ms, 40 frames of 10 000 points 30 us.
+// instead of 1755. 64 uneven trajectories 1.24 ms, 40 frames of 10 000 points 31 us.
 constexpr int SINGLE_THREADS = 128;
 __global__ void __launch_bounds__(SINGLE_THREADS, 16) k_tree_single(Ws w, int rows, int bidir) {
     pdl_wait();
