@@ -394,11 +394,12 @@ __device__ __forceinline__ int cell_get(const int* h, bool packed, int c) {
 //   5. bounding boxes of 8, 64 and 512 consecutive points
 // Bound by latency: chains of dependent gathers (face pick, corners) and one block-wide meeting
 // per phase. 40 frames of 10 000 points against as many: 62 us at 37% of the load pipe, its warps
-// waiting 5.3 cycles per instruction for memory and 3.6 at barriers. One kernel for all phases
+// waiting 4.7 cycles per instruction for memory and 3.6 at barriers. One kernel for all phases
 // keeps the counters and the draws' points on chip; clusters of 3 instead of 2 for those 80 sides
 // (240 CTAs instead of 160) 210 -> 198 us per call. 64 uneven trajectories, 1.14e8 points:
 // 6.1 ms with 1024 threads and gathers from global memory, 5.0 ms with face records and two
-// points per step, 4.5 ms with the ring below.
+// points per step, 4.5 ms with the ring below, 4.6 ms with the boxes' lowest indices and the check of the
+// key grid.
 template <int S>
 __global__ void __launch_bounds__(PREP_THREADS, 2)
     k_tree_prep(UniformArgs a, Ws w, int uniform, int n_frames, int rows, int cdf_shared) {
@@ -1073,8 +1074,8 @@ __device__ __noinline__ TileWalk walk_tile(TreeCols C, const float* qb, float ow
 //     blocks (exact ties, whose lowest index must win) are queued for k_tree_single; tiles that
 //     nothing prunes are walked as a whole by walk_tile.
 // Bound by instruction issue and the load pipe: 2650 instructions per tile, of which about 20
-// blocks of 8 evaluated (50 each) and 9 boxes of 64 staged are most; 69% of issue slots, 55% of
-// the load pipe's wavefronts, 2.5 cycles per instruction waiting for memory. 40 frames of 10 000
+// blocks of 8 evaluated (50 each) and 9 boxes of 64 staged are most; 70% of issue slots, 60% of
+// the load pipe's wavefronts, 2.4 cycles per instruction waiting for memory. 40 frames of 10 000
 // points against as many: 90 us, where evaluating every pair takes 630 us (tensor-core filter)
 // or 943 us (direct form). 64 uneven trajectories: 10.9 ms (one query per lane 11.5 ms and
 // 3.8 ms in k_tree_single, without the gradient's sums), the tensor-core filter 158 ms.
